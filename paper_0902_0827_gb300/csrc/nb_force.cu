@@ -50,6 +50,7 @@ struct ForceArgs {
     int *dbg_ij;
     long long dbg_cap;
     PairParams P;
+    PairConst2 C;             // packed constants of P
     // adjoint only
     const float4 *gslot;     // [S] dL/dF in sorted order (x, y, z, 0)
     const double *dLdE;      // [n_sys*2] dL/dE_LJ, dL/dE_C, or null
@@ -750,65 +751,138 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
 // same, each entry holds one tile (I, J).  Lane = jj + 8 ih holds j atom jj
 // of J and the i atoms ih and ih + 4 of I in registers, so every lane
 // computes two pairs of the 8 x 8 tile and the force on j is summed over only
-// 4 lanes; the i atoms' z-sorted lower half (pair A) and upper half (pair B)
-// are voted separately.  With one cluster per group the per-entry work is
-// per tile, but the i side needs no shared memory and the j-force sum is
-// short; which of this and the group kernel is faster depends on the system
-// (the autotuner measures it).
+// 4 lanes.  With one cluster per group the per-entry work is per tile, but
+// the i side needs no shared memory and the j-force sum is short; which of
+// this and the group kernel is faster depends on the system (the autotuner
+// measures it).
+//
+// The kernel is bound by instruction issue and register reads, not by the
+// FMA pipe (about half busy), so the two pairs of a lane share one
+// instruction: i atom ih in the low word and ih + 4 in the high word of
+// packed FP32 operations (pair_radial2), which round like the scalar ones.
+// A tile with a pair in range is evaluated whole; voting on its two halves
+// and skipping one (scalar code, 1.35 halves per tile) took 47.9 M warp
+// instructions and 63.4 us per launch at 23,500 atoms and 1,661 us at
+// 999,999; packed it is 40.3 M, 60.8 us and 1,621 us.  (An FMA with three
+// register operands, packed or not, issues at about 0.6 of its rate for the
+// register reads: the constants of the polynomials come from the parameter
+// bank and run at the full rate.)
 constexpr int kBatch1 = 32;  // entries staged per batch (one per lane)
 
-struct TileI {
-    float x, y, z, q;
-    int trow;
-    int orig;  // caller index (pair export)
+// The i cluster of a work unit for one lane: its atoms ih (low words) and
+// ih + 4 (high words).
+struct TileI2 {
+    f32x2 x, y, z, q;  // q: ke q
+    int trowA, trowB;  // type rows
+    int origA, origB;  // caller indices (pair export)
 };
 
-__device__ __forceinline__ TileI load_tile_i(const ForceArgs &A, long long slot, int T, bool debug)
+__device__ __forceinline__ TileI2 load_tile_i2(const ForceArgs &A, long long slot, int T, bool debug)
 {
-    float4 p = __ldg(A.xyzq + slot);
-    if (!is_real_coord(p.x)) p.x = p.y = p.z = kFarCoord;
-    TileI t;
-    t.x = p.x;
-    t.y = p.y;
-    t.z = p.z;
-    t.q = p.w * A.P.ke;
-    t.trow = __ldg(A.tslot + slot) * T;
-    t.orig = debug ? __ldg(A.perm + slot) : -1;
+    float4 p[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        p[k] = __ldg(A.xyzq + slot + 4 * k);
+        if (!is_real_coord(p[k].x)) p[k].x = p[k].y = p[k].z = kFarCoord;
+    }
+    TileI2 t;
+    t.x = pack2(p[0].x, p[1].x);
+    t.y = pack2(p[0].y, p[1].y);
+    t.z = pack2(p[0].z, p[1].z);
+    t.q = pack2(p[0].w * A.P.ke, p[1].w * A.P.ke);
+    t.trowA = __ldg(A.tslot + slot) * T;
+    t.trowB = __ldg(A.tslot + slot + 4) * T;
+    t.origA = debug ? __ldg(A.perm + slot) : -1;
+    t.origB = debug ? __ldg(A.perm + slot + 4) : -1;
     return t;
 }
 
-// Membership of one pair: the i atom at its image for the entry's shift code
-// (IMG: x_i - L on axes with code 2; the j side was shifted by the caller),
-// d = x_j - x_i and the FP32 predicate r2 < rc2.
-template <bool IMG>
-__device__ __forceinline__ bool tile1_member(const ForceArgs &A, const TileI &ti, uint32_t code, float4 pj, float Lx,
-                                             float Ly, float Lz, float &dx, float &dy, float &dz, float &r2)
+// Sums of a lane's two pairs over a work unit: the force on the i atoms and
+// the energies.
+struct Acc2 {
+    f32x2 fx, fy, fz, elj, ec;
+};
+
+// v where the lane's pair is inside the cutoff, else 0.
+__device__ __forceinline__ f32x2 masked2(f32x2 v, bool inA, bool inB)
 {
-    float ax = ti.x, ay = ti.y, az = ti.z;
-    if (IMG) {
-        if ((code & 3u) == 2u) ax = __fsub_rn(ax, Lx);
-        if (((code >> 2) & 3u) == 2u) ay = __fsub_rn(ay, Ly);
-        if ((code >> 4) == 2u) az = __fsub_rn(az, Lz);
-    }
-    r2 = disp_r2(pj.x, pj.y, pj.z, ax, ay, az, dx, dy, dz);
-    return r2 < A.P.rc2;
+    float a, b;
+    unpack2(v, a, b);
+    return pack2(inA ? a : 0.0f, inB ? b : 0.0f);
 }
 
+// Both pairs of a lane: -U'(r)/r of each (0 where masked), the energies added
+// to acc (the packed pair_fs).
+template <int RAD, bool W14>
+__device__ __forceinline__ f32x2 pair_fs2(const ForceArgs &A, const float4 *__restrict__ lj, const TileI2 &ti, bool inA,
+                                          bool inB, f32x2 r2, f32x2 qj, int tj, bool s14A, bool s14B, Acc2 &acc)
+{
+    const float2 *lj_lo = reinterpret_cast<const float2 *>(lj + A.P.n_types * A.P.n_types);
+    const int kA = ti.trowA + tj, kB = ti.trowB + tj;
+    const float4 abA = lj[kA], abB = lj[kB];
+    const float2 loA = lj_lo[kA], loB = lj_lo[kB];
+    const f32x2 qq = mul2(ti.q, qj);
+    f32x2 elj, frlj, ec, frc, r2inv;
+    if constexpr (RAD == 2) {
+        float rA2, rB2, qA, qB, ra, rb, ia, ib, e0, e1, l0, l1, c0, c1, f0, f1;
+        unpack2(r2, rA2, rB2);
+        unpack2(qq, qA, qB);
+        pair_rinv(rA2, ia, ra);
+        pair_rinv(rB2, ib, rb);
+        // (the tables' loads, not arithmetic, bound this: a half without a
+        // pair in range is skipped)
+        e0 = l0 = c0 = f0 = e1 = l1 = c1 = f1 = 0.0f;
+        if (__any_sync(kFull, inA)) pair_radial_tab(A.P, A.rtab, ra, abA.x, abA.y, loA, qA, e0, l0, c0, f0);
+        if (__any_sync(kFull, inB)) pair_radial_tab(A.P, A.rtab, rb, abB.x, abB.y, loB, qB, e1, l1, c1, f1);
+        elj = pack2(e0, e1);
+        frlj = pack2(l0, l1);
+        ec = pack2(c0, c1);
+        frc = pack2(f0, f1);
+        const f32x2 rinv = pack2(ia, ib);
+        r2inv = mul2(rinv, rinv);
+    } else {
+        pair_radial2<RAD == 1>(A.C, A.P, r2, abA, loA, abB, loB, qq, elj, frlj, ec, frc, r2inv);
+    }
+    f32x2 fs;
+    if (W14) {
+        const f32x2 wlj = pack2(s14A ? A.P.s14_lj : 1.0f, s14B ? A.P.s14_lj : 1.0f);
+        const f32x2 wc = pack2(s14A ? A.P.s14_c : 1.0f, s14B ? A.P.s14_c : 1.0f);
+        fs = mul2(fma2(wlj, frlj, mul2(wc, frc)), r2inv);
+        elj = mul2(wlj, elj);
+        ec = mul2(wc, ec);
+    } else {
+        fs = mul2(add2(frlj, frc), r2inv);
+    }
+    acc.elj = add2(acc.elj, masked2(elj, inA, inB));
+    acc.ec = add2(acc.ec, masked2(ec, inA, inB));
+    return masked2(fs, inA, inB);
+}
+
+// One entry (tile (I, J)) of a warp: the membership of the lane's two pairs,
+// their arithmetic packed (when any pair of the tile is in range), the force
+// on i added to acc, and the force on j summed over its 4 lanes.
 template <int RAD, bool VIRIAL, bool DEBUG, bool SPECIAL, bool IMG>
 __device__ __forceinline__ void tile1_entry(const ForceArgs &A, const float4 *__restrict__ lj, uint2 ent, float4 pj,
-                                            int tj, const TileI &ia, const TileI &ib, int jj, int ih, float Lx,
-                                            float Ly, float Lz, Acc &acA, Acc &acB, float (&wimg)[6], bool &ovf)
+                                            int tj, const TileI2 &ti, int jj, int ih, float Lx, float Ly, float Lz,
+                                            Acc2 &acc, float (&wimg)[3], bool &ovf)
 {
     const int J = (int)(ent.x & kJMask);
     const uint32_t code = IMG ? (ent.x >> kShiftBit) & 0x3Fu : 0u;
-    if (IMG) {  // j-side images (code 1): fl(x_j - L), as the other kernels stage them
+    f32x2 ix = ti.x, iy = ti.y, iz = ti.z;
+    if (IMG) {  // code 1: fl(x_j - L) on the j side, code 2: fl(x_i - L) on the i side
         if ((code & 3u) == 1u) pj.x = __fsub_rn(pj.x, Lx);
         if (((code >> 2) & 3u) == 1u) pj.y = __fsub_rn(pj.y, Ly);
         if ((code >> 4) == 1u) pj.z = __fsub_rn(pj.z, Lz);
+        if ((code & 3u) == 2u) ix = sub2(ix, pack2(Lx, Lx));
+        if (((code >> 2) & 3u) == 2u) iy = sub2(iy, pack2(Ly, Ly));
+        if ((code >> 4) == 2u) iz = sub2(iz, pack2(Lz, Lz));
     }
-    float dxA, dyA, dzA, r2A, dxB, dyB, dzB, r2B;
-    bool inA = tile1_member<IMG>(A, ia, code, pj, Lx, Ly, Lz, dxA, dyA, dzA, r2A);
-    bool inB = tile1_member<IMG>(A, ib, code, pj, Lx, Ly, Lz, dxB, dyB, dzB, r2B);
+    // e = x_i - x_j = -d; r2 as disp_r2
+    const f32x2 ex = sub2(ix, pack2(pj.x, pj.x)), ey = sub2(iy, pack2(pj.y, pj.y)), ez = sub2(iz, pack2(pj.z, pj.z));
+    f32x2 r2 = fma2(ez, ez, fma2(ey, ey, mul2(ex, ex)));
+    float r2A, r2B;
+    unpack2(r2, r2A, r2B);
+    bool inA = r2A < A.P.rc2, inB = r2B < A.P.rc2;
     bool s14A = false, s14B = false;
     if (SPECIAL) {  // exclusion bitmask of the tile: bit 8 i + j
         const ulonglong2 m = A.gmask[ent.y >> kMaskSlotBit];  // records of one cluster
@@ -817,46 +891,68 @@ __device__ __forceinline__ void tile1_entry(const ForceArgs &A, const float4 *__
         inB = inB && !((m.x >> bB) & 1ull);
         s14A = (m.y >> bA) & 1ull;
         s14B = (m.y >> bB) & 1ull;
+        // only a flagged tile can hold r2 = 0 (the self tile's diagonal, masked)
+        r2 = pack2(inA ? r2A : 1.0f, inB ? r2B : 1.0f);
     }
-    const bool anyA = __any_sync(kFull, inA), anyB = __any_sync(kFull, inB);
-    if (DEBUG) count_tile(A, anyA, anyB);
-    if (!anyA && !anyB) return;
-    const int jorig = DEBUG ? __ldg(A.perm + (long long)J * kCluster + jj) : -1;
-    float fjx = 0.0f, fjy = 0.0f, fjz = 0.0f;
-    if (anyA) {
-        if (DEBUG && inA) record_pair(A, ia.orig, jorig);
-        // only a special (flagged) tile can hold r2 = 0 (the self tile's diagonal, masked)
-        eval_pair<RAD, SPECIAL>(A.P, lj, A.rtab, ia.trow, ia.q, inA, dxA, dyA, dzA, SPECIAL ? (inA ? r2A : 1.0f) : r2A,
-                                pj.w, tj, s14A, acA, fjx, fjy, fjz);
+    if (DEBUG) count_tile(A, __any_sync(kFull, inA), __any_sync(kFull, inB));
+    if (!__any_sync(kFull, inA || inB)) return;
+    if (DEBUG) {
+        const int jorig = __ldg(A.perm + (long long)J * kCluster + jj);
+        if (inA) record_pair(A, ti.origA, jorig);
+        if (inB) record_pair(A, ti.origB, jorig);
     }
-    if (anyB) {
-        if (DEBUG && inB) record_pair(A, ib.orig, jorig);
-        eval_pair<RAD, SPECIAL>(A.P, lj, A.rtab, ib.trow, ib.q, inB, dxB, dyB, dzB, SPECIAL ? (inB ? r2B : 1.0f) : r2B,
-                                pj.w, tj, s14B, acB, fjx, fjy, fjz);
-    }
-    // the force on j atom jj: sum over its 4 lanes, then lanes ih = 0, 1, 2
-    // add the x, y, z components
-#pragma unroll
-    for (int o = 8; o < 32; o <<= 1) {
-        fjx = __fadd_rn(fjx, __shfl_xor_sync(kFull, fjx, o));
-        fjy = __fadd_rn(fjy, __shfl_xor_sync(kFull, fjy, o));
-        fjz = __fadd_rn(fjz, __shfl_xor_sync(kFull, fjz, o));
-    }
-    const float fc = ih == 0 ? fjx : (ih == 1 ? fjy : fjz);
-    const long long fv = tile_fixed(fc, ovf);  // every lane (lane ih = 3 holds z again): no branch
+    const f32x2 fs = pair_fs2<RAD, SPECIAL>(A, lj, ti, inA, inB, r2, pack2(pj.w, pj.w), tj, s14A, s14B, acc);
+    acc.fx = fma2(fs, ex, acc.fx);  // F_i = fs e
+    acc.fy = fma2(fs, ey, acc.fy);
+    acc.fz = fma2(fs, ez, acc.fz);
+    // F_j = -fs e: both pairs, then the 4 lanes of j atom jj (ih = 0..3) as
+    // (0 + 1) + (2 + 3).  The lanes trade components instead of all summing
+    // all three: lanes ih = 0, 1, 2 end with x, y, z (ih = 3 with y again).
+    float fA, fB, e0, e1, fj[3];
+    unpack2(fs, fA, fB);
+    unpack2(ex, e0, e1);
+    fj[0] = __fmaf_rn(fB, -e1, __fmul_rn(fA, -e0));
+    unpack2(ey, e0, e1);
+    fj[1] = __fmaf_rn(fB, -e1, __fmul_rn(fA, -e0));
+    unpack2(ez, e0, e1);
+    fj[2] = __fmaf_rn(fB, -e1, __fmul_rn(fA, -e0));
+    const bool odd = ih & 1, upper = ih & 2;
+    const float xy = __fadd_rn(odd ? fj[1] : fj[0], __shfl_xor_sync(kFull, odd ? fj[0] : fj[1], 8));
+    const float zz = __fadd_rn(fj[2], __shfl_xor_sync(kFull, fj[2], 8));
+    const bool take_z = upper && !odd;
+    const float fc = __fadd_rn(take_z ? zz : xy, __shfl_xor_sync(kFull, odd || upper ? xy : zz, 16));
+    const long long fv = tile_fixed(fc, ovf);  // every lane: no branch
     if (ih < 3) atomicAdd((unsigned long long *)&A.facc[24ll * J + 3 * jj + ih], (unsigned long long)fv);
-    if (VIRIAL && IMG && ih == 0) {
+    if (VIRIAL && IMG) {
+        // periodic-image part of the virial, s (x) f_j with the entry's shift
+        // s of j: lane ih < 3 holds s_x, s_y, s_z times component ih
         const uint32_t cx = code & 3u, cy = (code >> 2) & 3u, cz = code >> 4;
         const float sx = cx == 1u ? -Lx : (cx == 2u ? Lx : 0.0f);
         const float sy = cy == 1u ? -Ly : (cy == 2u ? Ly : 0.0f);
         const float sz = cz == 1u ? -Lz : (cz == 2u ? Lz : 0.0f);
-        wimg[0] = __fmaf_rn(sx, fjx, wimg[0]);
-        wimg[1] = __fmaf_rn(sy, fjy, wimg[1]);
-        wimg[2] = __fmaf_rn(sz, fjz, wimg[2]);
-        wimg[3] = __fmaf_rn(sx, fjy, wimg[3]);
-        wimg[4] = __fmaf_rn(sx, fjz, wimg[4]);
-        wimg[5] = __fmaf_rn(sy, fjz, wimg[5]);
+        wimg[0] = __fmaf_rn(sx, fc, wimg[0]);
+        wimg[1] = __fmaf_rn(sy, fc, wimg[1]);
+        wimg[2] = __fmaf_rn(sz, fc, wimg[2]);
     }
+}
+
+// The image virial of a work unit (FP32 per lane, see tile1_entry) to the
+// warp's fixed-point sums (2^20): lane k < 6 holds component k (xx, yy, zz,
+// xy, xz, yz) in wv.  Rounded per lane and unit, so the sums do not depend on
+// which warp took which unit.
+__device__ __forceinline__ void tile1_virial_unit(float (&wimg)[3], long long &wv, int lane)
+{
+    const int ih = lane >> 3;
+    // the component of s and of f (its lane ih) of each virial component
+    constexpr int ks[6] = {0, 1, 2, 0, 0, 1}, kf[6] = {0, 1, 2, 1, 2, 2};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        long long x = ih == kf[k] ? __float2ll_rn(wimg[ks[k]] * (float)kVirScale) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+        if (lane == k) wv += x;
+    }
+    wimg[0] = wimg[1] = wimg[2] = 0.0f;
 }
 
 __host__ __device__ inline size_t tile1_warp_bytes() { return (size_t)kBatch1 * kCluster * (16 + 4); }
@@ -883,7 +979,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
     int cur_sys = -1;
     float Lx = 0.0f, Ly = 0.0f, Lz = 0.0f;
     long long esum[2] = {0, 0};
-    float wimg[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    float wimg[3] = {0.0f, 0.0f, 0.0f};
     long long wv = 0;
     bool ovf = false;
     int u = 0;
@@ -899,8 +995,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
         const int I = U.g;
         const int sys_id = __ldg(A.clus_sys + I);
         const long long s0 = (long long)I * kCluster;
-        const TileI ia = load_tile_i(A, s0 + ih, T, DEBUG);
-        const TileI ib = load_tile_i(A, s0 + ih + 4, T, DEBUG);
+        const TileI2 ti = load_tile_i2(A, s0 + ih, T, DEBUG);
         const uint2 *row = A.glist + U.base;
         const uint2 first = lane < A.cap / kListSegs ? __ldg(row + lane) : make_uint2(0u, 0u);
         if (U.e_begin < U.e_end) {
@@ -917,7 +1012,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                 Ly = A.sys[sys_id].L[1];
                 Lz = A.sys[sys_id].L[2];
             }
-            Acc acA = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, acB = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            Acc2 acc = {0ull, 0ull, 0ull, 0ull, 0ull};
             bool unit_img = false;
             for (int e0 = U.e_begin; e0 < U.e_end; e0 += kBatch1) {
                 const int ne = min(kBatch1, U.e_end - e0);
@@ -942,8 +1037,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                     const int k = __ffs(plain) - 1;
                     plain &= plain - 1u;
                     const uint2 ent = make_uint2(__shfl_sync(kFull, my.x, k), __shfl_sync(kFull, my.y, k));
-                    tile1_entry<RAD, VIRIAL, DEBUG, false, false>(A, lj, ent, sjp[swz(k, jj)], sjt[swz(k, jj)], ia, ib,
-                                                                  jj, ih, Lx, Ly, Lz, acA, acB, wimg, ovf);
+                    tile1_entry<RAD, VIRIAL, DEBUG, false, false>(A, lj, ent, sjp[swz(k, jj)], sjt[swz(k, jj)], ti, jj, ih, Lx, Ly, Lz, acc, wimg, ovf);
                 }
                 while (other) {
                     const int k = __ffs(other) - 1;
@@ -955,14 +1049,11 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                     const bool special = (ent.x & kExclFlag) != 0u;
                     if (img) {
                         if (special)
-                            tile1_entry<RAD, VIRIAL, DEBUG, true, true>(A, lj, ent, pj, tj, ia, ib, jj, ih, Lx, Ly, Lz,
-                                                                        acA, acB, wimg, ovf);
+                            tile1_entry<RAD, VIRIAL, DEBUG, true, true>(A, lj, ent, pj, tj, ti, jj, ih, Lx, Ly, Lz, acc, wimg, ovf);
                         else
-                            tile1_entry<RAD, VIRIAL, DEBUG, false, true>(A, lj, ent, pj, tj, ia, ib, jj, ih, Lx, Ly,
-                                                                         Lz, acA, acB, wimg, ovf);
+                            tile1_entry<RAD, VIRIAL, DEBUG, false, true>(A, lj, ent, pj, tj, ti, jj, ih, Lx, Ly, Lz, acc, wimg, ovf);
                     } else {
-                        tile1_entry<RAD, VIRIAL, DEBUG, true, false>(A, lj, ent, pj, tj, ia, ib, jj, ih, Lx, Ly, Lz,
-                                                                     acA, acB, wimg, ovf);
+                        tile1_entry<RAD, VIRIAL, DEBUG, true, false>(A, lj, ent, pj, tj, ti, jj, ih, Lx, Ly, Lz, acc, wimg, ovf);
                     }
                 }
                 __syncwarp();  // the staging buffer is rewritten by the next batch
@@ -970,7 +1061,10 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
             // force on the i atoms: the 8 lanes of each atom summed in FP32
             // (a fixed butterfly), then lanes jj < 3 add atom ih, jj = 3..5
             // atom ih + 4 in fixed point
-            float v[6] = {acA.fx, acA.fy, acA.fz, acB.fx, acB.fy, acB.fz};
+            float v[6];
+            unpack2(acc.fx, v[0], v[3]);
+            unpack2(acc.fy, v[1], v[4]);
+            unpack2(acc.fz, v[2], v[5]);
 #pragma unroll
             for (int o = 1; o < 8; o <<= 1)
 #pragma unroll
@@ -983,9 +1077,12 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                 const long long slot = s0 + ih + (jj < 3 ? 0 : 4);
                 atomicAdd((unsigned long long *)&A.facc[3 * slot + (jj < 3 ? jj : jj - 3)], (unsigned long long)fi);
             }
-            esum[0] += tile_fixed(acA.elj, ovf) + tile_fixed(acB.elj, ovf);
-            esum[1] += tile_fixed(acA.ec, ovf) + tile_fixed(acB.ec, ovf);
-            if (VIRIAL && unit_img) tile_virial_unit(wimg, wv, lane);
+            float eA, eB;
+            unpack2(acc.elj, eA, eB);
+            esum[0] += tile_fixed(eA, ovf) + tile_fixed(eB, ovf);
+            unpack2(acc.ec, eA, eB);
+            esum[1] += tile_fixed(eA, ovf) + tile_fixed(eB, ovf);
+            if (VIRIAL && unit_img) tile1_virial_unit(wimg, wv, lane);
             if (__any_sync(kFull, ovf)) {
                 if (lane == 0) atomicOr(A.status, ST_OVERFLOW);
                 ovf = false;
@@ -1713,6 +1810,35 @@ static void launch_force_t(nb_ctx *ctx, const ForceArgs &A, bool beside_pme, boo
     }
 }
 
+// The packed constants of a parameter block.
+static PairConst2 make_const2(const PairParams &P)
+{
+    auto twice = [](float v) {
+        uint32_t b;
+        memcpy(&b, &v, sizeof(b));
+        return (f32x2)b << 32 | b;
+    };
+    PairConst2 C;
+    C.rc2 = twice(P.rc2);
+    C.rs2 = twice(P.rs2);
+    C.sw_a = twice(P.sw_a);
+    C.sw_b = twice(P.sw_b);
+    C.neg_sw_c = twice(-P.sw_c);
+    C.neg_alpha_half = twice(-P.alpha_half);
+    C.a2_hi = twice(P.neg_a2_log2e);
+    C.neg_a2_hi = twice(-P.neg_a2_log2e);
+    C.neg_a2_lo = twice(-P.neg_a2_log2e_lo);
+    C.two_a_sqpi = twice(P.two_a_sqpi);
+    C.magic = twice(12582912.0f);
+    C.one = twice(1.0f);
+    C.neg_one = twice(-1.0f);
+    C.neg_half = twice(-0.5f);
+    C.neg_zero = twice(-0.0f);
+    for (int k = 0; k <= kErfcDeg; ++k) C.erfc_c[k] = twice(P.erfc_c[k]);
+    for (int k = 0; k <= kExp2Deg; ++k) C.exp2_c[k] = twice(P.exp2_c[k]);
+    return C;
+}
+
 static ForceArgs make_args(nb_ctx *ctx)
 {
     auto &d = ctx->d;
@@ -1739,6 +1865,7 @@ static ForceArgs make_args(nb_ctx *ctx)
     A.dbg_ij = d.dbg_ij;
     A.dbg_cap = d.dbg_cap;
     A.P = ctx->pp;
+    A.C = make_const2(ctx->pp);
     return A;
 }
 

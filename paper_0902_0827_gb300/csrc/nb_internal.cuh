@@ -104,6 +104,22 @@ struct PairParams {
     int tab_n;           // intervals of the tables (0: direct evaluation)
 };
 
+// The constants of the packed pair arithmetic (pair_radial2), each twice in
+// one 64-bit word: an operand of fma.rn.f32x2 and the like.  Signs are chosen
+// so that no operand has to be negated.
+using f32x2 = unsigned long long;
+struct PairConst2 {
+    f32x2 rc2, rs2;
+    f32x2 sw_a, sw_b, neg_sw_c;
+    f32x2 neg_alpha_half;
+    f32x2 a2_hi, neg_a2_hi, neg_a2_lo;  // c = -alpha^2 log2(e) as hi + lo: hi, -hi, -lo
+    f32x2 two_a_sqpi;
+    f32x2 magic;                        // 1.5 2^23
+    f32x2 one, neg_one, neg_half, neg_zero;
+    f32x2 erfc_c[kErfcDeg + 1];
+    f32x2 exp2_c[kExp2Deg + 1];
+};
+
 struct DevBuffers {
     SysDesc *sys = nullptr;          // [n_sys]
     int *atom_sys = nullptr;         // [N]
