@@ -1601,28 +1601,60 @@ __global__ void k_pack(int slot_cap, const int *__restrict__ counts, const int *
     tslot[s] = t;
 }
 
-// Add a warp's per-lane fixed-point virial terms (lanes with sys < 0 hold
-// none) to the per-system sums: one reduction and 6 atomics per distinct
-// system among the lanes, into the block's shared sums when the system is
-// the block's (blk_sys), else straight to global memory.
-__device__ __forceinline__ void flush_virial_warp(long long *w, int sys, long long *sys_acc, int blk_sys,
-                                                  unsigned long long *blk_w)
+// x v 2^-12 rounded to the nearest integer (half up), for a wrapped
+// coordinate x >= 0 and a fixed-point force v (2^32): a virial term on the
+// 2^20 grid.  Exact in integers, mantissa times v with one rounding: the
+// FP64 unit would take 64 cycles per warp for each of the products and
+// conversions (15 per atom).
+// (beyond 2,048 A the product does not fit and FP64 takes over, in a function
+// of its own: inlined, the compiler ran both sides for every atom)
+__device__ __noinline__ long long virial_term_fp64(float x, long long v)
 {
+    return __double2ll_rn((double)x * ((double)v * (kVirScale / kFixScale)));
+}
+
+__device__ __forceinline__ long long virial_term(float x, long long v)
+{
+    const unsigned b = __float_as_uint(x);
+    const int e = (int)(b >> 23);
+    if (e > 137) return virial_term_fp64(x, v);  // x >= 2048
+    const unsigned m = e > 0 ? (b & 0x7FFFFFu) | 0x800000u : 0u;  // x = m 2^(e - 150); subnormal: no term
+    const long long hi = v >> 24;
+    const unsigned lo = (unsigned)v & 0xFFFFFFu;
+    // m v = q 2^24 + (a remainder that floor and half up never see)
+    const long long q = (long long)m * hi + (long long)(((unsigned long long)m * lo) >> 24);
+    const int sh = min(138 - e, 62);  // 24 + sh = 150 - e + 12
+    return (q + (1ll << (sh - 1))) >> sh;
+}
+
+constexpr int kUnpackThreads = 64;  // 64 threads of at most 64 registers: what the force kernel's 24 warps of 80 leave
+
+// Add a warp's per-lane virial terms (lanes with sys < 0 hold none) to the
+// per-system sums: for each distinct system among the lanes one reduction in
+// which the lanes trade components (8 to 4 to 2 to 1 per lane, then two more
+// levels), and one atomic per component.
+__device__ __forceinline__ void flush_virial_warp(long long (&w)[6], int sys, long long *sys_acc)
+{
+    const int lane = threadIdx.x & 31;
     unsigned rem = __ballot_sync(kFull, sys >= 0);
     while (rem) {
-        const int leader = __ffs(rem) - 1;
-        const int cs = __shfl_sync(kFull, sys, leader);
+        const int cs = __shfl_sync(kFull, sys, __ffs(rem) - 1);
         const bool mine = sys == cs;
+        long long v[8];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            long long x = mine ? w[k] : 0;
+        for (int k = 0; k < 8; ++k) v[k] = k < 6 && mine ? w[k] : 0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-            if ((int)(threadIdx.x & 31) == leader) {
-                if (cs == blk_sys) atomicAdd(&blk_w[k], (unsigned long long)x);
-                else atomicAdd((unsigned long long *)&sys_acc[cs * kTaskVals + 2 + k], (unsigned long long)x);
+        for (int n = 4; n >= 1; n >>= 1) {  // lane bit n set: keep the upper n components
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                const long long keep = lane & n ? v[k + n] : v[k], give = lane & n ? v[k] : v[k + n];
+                v[k] = keep + __shfl_xor_sync(kFull, give, n);
             }
         }
+        v[0] += __shfl_xor_sync(kFull, v[0], 8);
+        v[0] += __shfl_xor_sync(kFull, v[0], 16);
+        // lane k < 8 holds component k
+        if (lane < 6 && v[0]) atomicAdd((unsigned long long *)&sys_acc[cs * kTaskVals + 2 + lane], (unsigned long long)v[0]);
         rem &= ~__ballot_sync(kFull, mine);
     }
 #pragma unroll
@@ -1636,77 +1668,74 @@ __device__ __forceinline__ void flush_virial_warp(long long *w, int sys, long lo
 // W_ab = sum_pairs d_a f_b (d = x_j' - x_i, f the force on j) equals
 // sum_atoms x_a F_b over the wrapped coordinates x and total forces F, plus
 // the periodic-image terms added by the force kernel.  Each atom's terms are
-// rounded to the 2^20 fixed-point grid in FP64 and summed as integers per
-// thread (grid-stride loop, atoms in system order) and per warp.
+// rounded to the 2^20 fixed-point grid and summed as integers per thread
+// (grid-stride loop, atoms in system order) and per warp.
+//
+// Latency bound at 23,500 atoms, memory bound at 1 M (about 100 bytes an
+// atom in scattered 32-byte sectors).  Blocks of 64 threads fit beside the
+// force kernel's warps, so most are resident when it ends; a thread's slot
+// and position (complete before the force kernel began) are loaded before
+// the wait; the arithmetic is integer.  With blocks of 256 threads and FP64
+// products the kernel took 53 us at 999,999 atoms, now 25 us (ncu, cold);
+// rebuild + forces 89.5 -> 85.6 us at 23,500 atoms, 52.2 -> 48.6 us at 6,144,
+// 2173 -> 2129 us at 999,999.
 template <bool VIRIAL>
-__global__ void __launch_bounds__(256) k_unpack_forces(int n_atoms, int *__restrict__ counts,
-                                                       const int *__restrict__ inv, const long long *__restrict__ facc,
-                                                       float *__restrict__ F, const float4 *__restrict__ xyzq,
-                                                       const int *__restrict__ atom_sys, long long *__restrict__ sys_acc,
-                                                       int n_sys, double *__restrict__ energy, double *__restrict__ virial,
-                                                       const long long *__restrict__ pme_f,
-                                                       const long long *__restrict__ pme_s, double pme_self)
+__global__ void __launch_bounds__(kUnpackThreads, 16)
+    k_unpack_forces(int n_atoms, int *__restrict__ counts, const int *__restrict__ inv, const long long *__restrict__ facc,
+                    float *__restrict__ F, const float4 *__restrict__ xyzq, const int *__restrict__ atom_sys,
+                    long long *__restrict__ sys_acc, int n_sys, double *__restrict__ energy,
+                    double *__restrict__ virial, const long long *__restrict__ pme_f,
+                    const long long *__restrict__ pme_s, double pme_self)
 {
+    const int stride = gridDim.x * blockDim.x;
+    int a = blockIdx.x * blockDim.x + threadIdx.x;
+    // of the kernels before the force kernel
+    int s = a < n_atoms ? inv[a] : -1;
+    float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    int sys = -1;
+    if (VIRIAL && s >= 0) {
+        x = xyzq[s];
+        sys = n_sys == 1 ? 0 : atom_sys[a];
+    }
     pdl_entry();
     long long w[6] = {0, 0, 0, 0, 0, 0};
     int wsys = -1;
-    __shared__ unsigned long long blk_w[6];
-    __shared__ int blk_sys;
-    if (VIRIAL) {
-        if (threadIdx.x < 6) blk_w[threadIdx.x] = 0ull;
-        if (threadIdx.x == 0) {
-            const int a0 = blockIdx.x * blockDim.x;
-            blk_sys = a0 < n_atoms ? atom_sys[a0] : -1;
+    for (int a0 = a - (int)threadIdx.x; a0 < n_atoms; a0 += stride) {
+        if (VIRIAL) {
+            // atoms come in system order: flush a lane's sums before it moves on
+            if (__any_sync(kFull, sys >= 0 && wsys >= 0 && sys != wsys)) {
+                flush_virial_warp(w, wsys, sys_acc);
+                wsys = -1;
+            }
         }
-        __syncthreads();
-    }
-    for (int a0 = blockIdx.x * blockDim.x; a0 < n_atoms; a0 += gridDim.x * blockDim.x) {
-        const int a = a0 + threadIdx.x;
-        const int s = a < n_atoms ? inv[a] : -1;
-        int sys = -1;
-        long long c[6];
         if (s >= 0) {
             const long long v0 = facc[3ll * s], v1 = facc[3ll * s + 1], v2 = facc[3ll * s + 2];
-            const float sc = 2.3283064365386963e-10f;  // 2^-32
             // PME forces (same slot order) join the sum before the one
             // rounding; the atom part of the virial is the short-range forces' alone
             const long long p0 = pme_f ? pme_f[3ll * s] : 0, p1 = pme_f ? pme_f[3ll * s + 1] : 0,
                             p2 = pme_f ? pme_f[3ll * s + 2] : 0;
-            F[3ll * a] = __ll2float_rn(v0 + p0) * sc;
-            F[3ll * a + 1] = __ll2float_rn(v1 + p1) * sc;
-            F[3ll * a + 2] = __ll2float_rn(v2 + p2) * sc;
+            F[3ll * a] = fixed_to_float(v0 + p0);
+            F[3ll * a + 1] = fixed_to_float(v1 + p1);
+            F[3ll * a + 2] = fixed_to_float(v2 + p2);
             if (VIRIAL) {
-                const double r = kVirScale / kFixScale;
-                const double fx = (double)v0 * r, fy = (double)v1 * r, fz = (double)v2 * r;
-                const float4 x = xyzq[s];
-                c[0] = __double2ll_rn(x.x * fx);
-                c[1] = __double2ll_rn(x.y * fy);
-                c[2] = __double2ll_rn(x.z * fz);
-                c[3] = __double2ll_rn(x.x * fy);
-                c[4] = __double2ll_rn(x.x * fz);
-                c[5] = __double2ll_rn(x.y * fz);
-                sys = atom_sys[a];
-            }
-        }
-        if (VIRIAL) {
-            // atoms come in system order: flush a lane's sums before it moves on
-            if (__any_sync(kFull, sys >= 0 && wsys >= 0 && sys != wsys)) {
-                flush_virial_warp(w, wsys, sys_acc, blk_sys, blk_w);
-                wsys = -1;
-            }
-            if (sys >= 0) {
+                w[0] += virial_term(x.x, v0);
+                w[1] += virial_term(x.y, v1);
+                w[2] += virial_term(x.z, v2);
+                w[3] += virial_term(x.x, v1);
+                w[4] += virial_term(x.x, v2);
+                w[5] += virial_term(x.y, v2);
                 wsys = sys;
-#pragma unroll
-                for (int k = 0; k < 6; ++k) w[k] += c[k];
             }
         }
+        a += stride;
+        s = a < n_atoms ? inv[a] : -1;
+        sys = -1;
+        if (VIRIAL && s >= 0) {
+            x = xyzq[s];
+            sys = n_sys == 1 ? 0 : atom_sys[a];
+        }
     }
-    if (VIRIAL) {
-        flush_virial_warp(w, wsys, sys_acc, blk_sys, blk_w);
-        __syncthreads();
-        if (threadIdx.x < 6 && blk_sys >= 0 && blk_w[threadIdx.x])
-            atomicAdd((unsigned long long *)&sys_acc[blk_sys * kTaskVals + 2 + threadIdx.x], blk_w[threadIdx.x]);
-    }
+    if (VIRIAL) flush_virial_warp(w, wsys, sys_acc);
     if (!energy && !virial) return;
     // the last block to finish converts the per-system sums (counts[2] is the
     // completion ticket: zero on entry, reset here)
@@ -1748,13 +1777,12 @@ __global__ void k_unpack_adjoint(int slot_cap, const int *__restrict__ counts, c
     if (s >= slot_cap || s >= counts[0]) return;
     const int a = perm[s];
     if (a < 0) return;
-    const float sc = 2.3283064365386963e-10f;  // 2^-32
     if (dpos) {
-        dpos[3ll * a] = __ll2float_rn(gacc[4ll * s]) * sc;
-        dpos[3ll * a + 1] = __ll2float_rn(gacc[4ll * s + 1]) * sc;
-        dpos[3ll * a + 2] = __ll2float_rn(gacc[4ll * s + 2]) * sc;
+        dpos[3ll * a] = fixed_to_float(gacc[4ll * s]);
+        dpos[3ll * a + 1] = fixed_to_float(gacc[4ll * s + 1]);
+        dpos[3ll * a + 2] = fixed_to_float(gacc[4ll * s + 2]);
     }
-    if (dq) dq[a] = __ll2float_rn(gacc[4ll * s + 3]) * sc;
+    if (dq) dq[a] = fixed_to_float(gacc[4ll * s + 3]);
 }
 
 // Kernel function attributes belong to each device's context, so the
@@ -1984,9 +2012,9 @@ cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, doub
         if (e != cudaSuccess) return e;
     }
     if (d_F) {  // else the caller's next kernel reads the fixed-point sums (the MD step)
-        const int tb = 256;
+        const int tb = kUnpackThreads;
         const int S = (int)ctx->n_atoms;
-        const int blocks = std::max(1, std::min((S + tb - 1) / tb, 4 * ctx->num_sms));
+        const int blocks = std::max(1, std::min((S + tb - 1) / tb, 16 * ctx->num_sms));
         double *en = debug_pairs ? nullptr : d_energy;
         double *vi = debug_pairs ? nullptr : d_virial;
         const long long *pf = pme ? pme_forces_acc(ctx) : nullptr, *ps = pme ? pme_sums_acc(ctx) : nullptr;

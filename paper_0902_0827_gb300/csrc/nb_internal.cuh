@@ -222,6 +222,22 @@ __device__ __forceinline__ float wrap_coord(float x, float L)
     return x;
 }
 
+// A fixed-point value (2^32) as the nearest FP32, the bits of
+// __ll2float_rn(v) * 2^-32.  The 64-bit conversions run on the FP64 unit
+// here, one warp in 64 cycles per SM sub-partition (measured: 0.015 warp
+// instructions per cycle, 0.12 for the 32-bit ones); this takes about 14
+// integer instructions and one 32-bit conversion: the leading 32 bits, the
+// others ORed into the lowest one so that the rounding sees them.
+__device__ __forceinline__ float fixed_to_float(long long v)
+{
+    const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = min(__clzll((long long)u), 63);
+    const unsigned long long n = u << lz;
+    const unsigned hi = (unsigned)(n >> 32) | ((unsigned)n != 0u ? 1u : 0u);
+    const float f = __uint2float_rn(hi) * __int_as_float((127 - lz) << 23);  // 2^-lz: exact
+    return v < 0 ? -f : f;
+}
+
 // Programmatic dependent launch.  Every kernel of the library calls
 // pdl_entry() before it reads or writes anything that another kernel writes
 // (at its start, or after a prologue that only fills shared memory from
