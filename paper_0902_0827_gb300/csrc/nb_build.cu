@@ -433,9 +433,12 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
         bb[2 * I + 1] = make_float4(hx, hy, hz, 0.0f);
         clus_sys[I] = col_sys[c];
         // i-groups: runs of `group` consecutive clusters of the column
-        const int gi = col_grp[c] + q / group;
-        clus_grp[I] = gi;
-        if (q % group == 0) grp[gi] = make_int2(I, min(group, nclus - q));
+        // (groups of one are numbered like their clusters: no table)
+        if (group != 1) {
+            const int gi = col_grp[c] + q / group;
+            clus_grp[I] = gi;
+            if (q % group == 0) grp[gi] = make_int2(I, min(group, nclus - q));
+        }
     }
     __syncthreads();
     // z-bin index: for b = 0..nzb, (first cluster with z_hi >= b dz, first
@@ -599,11 +602,11 @@ __device__ __forceinline__ int div_small(int a, int b, float inv_b, int &r)
     return q;
 }
 
-// A4: i-group lists, one warp per group of up to 8 consecutive clusters of a
-// column (clusters c0 .. c0 + n - 1), kGListWarps groups per block.  The
-// columns within reach of the group's bounding box (with periodic images)
-// are scanned in order.  Clusters of a column are
-// z-sorted, so the ones whose z-range (under the z images -L, 0, +L,
+// A4: i-group lists (groups of 4 or 8 clusters; k_glist1 below serves groups
+// of one), one warp per group of up to 8 consecutive clusters of a column
+// (clusters c0 .. c0 + n - 1), kGListWarps groups per block.  The columns
+// within reach of the group's bounding box (with periodic images) are scanned
+// in order.  Clusters of a column are z-sorted, so the ones whose z-range (under the z images -L, 0, +L,
 // concatenated as virtual indices -nj..2nj-1) comes within the cutoff of the
 // group form one window per column; the windows of 32 columns are flattened
 // and every candidate (J, image) gets the mask of the group clusters whose
@@ -665,9 +668,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
     pdl_entry();
     if (g >= A.counts[4]) return;  // the whole warp
     const unsigned lt = (1u << lane) - 1u;
-    // one-cluster groups are numbered like their clusters (the scans of
-    // cluster and group counts per column coincide): no load
-    const int2 gr = A.group == 1 ? make_int2(g, 1) : A.grp[g];
+    const int2 gr = A.grp[g];
     const int c0 = gr.x, n = gr.y, K = A.K;
     __shared__ float4 s_lo_all[kGListWarps][kMaxGroup], s_hi_all[kGListWarps][kMaxGroup];
     __shared__ int s_col_all[kGListWarps][32];
@@ -689,11 +690,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
     __syncwarp();
     const int np = kCluster * n * K;
     const float inv_K = 1.0f / (float)K;
-    bool full = false;
-    // groups of one cluster (8 K <= 128 partner entries, one batch): every
-    // lane keeps its entries (partner cluster << 7 | is14 << 6 | bit 8 a + jj)
-    // for the warp-cooperative masks
-    int pk[kPartnerBatch] = {-1, -1, -1, -1};  // the partner table overflowed: flag every entry
+    bool full = false;  // the partner table overflowed: flag every entry
     for (int t0 = 0; t0 < np; t0 += kPartnerBatch * 32) {
         // the three dependent loads of kPartnerBatch rounds at a time
         int pv[kPartnerBatch];
@@ -724,8 +721,6 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
                 const int a = div_small(t, K, inv_K, rr);  // group atom of entry t
                 if (hs < 0) full = true;
                 else s_link[t] = (atomicExch(&s_head[hs], t) & kLinkEnd) | (a << 16);
-                if (t0 == 0 && A.group == 1)
-                    pk[r] = (((pv[r] >> 1) / kCluster) << 7) | ((pv[r] & 1) << 6) | (a * kCluster + ((pv[r] >> 1) & 7));
             }
         }
     }
@@ -850,17 +845,13 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
                 int hs = -1;
                 bool flag = false;
                 if (J[h] >= 0 && box_gap2(lo, hi, jl[h], jh[h]) < rcm2) {
-                    const int gJ = A.group == 1 ? J[h] : A.clus_grp[J[h]];  // groups of one cluster: the same index
+                    const int gJ = A.clus_grp[J[h]];
                     const bool other = gJ != g;
                     if (!other || keep_groups(g, gJ)) {
-                        if (n == 1) {
-                            cm = other || keep_in_group(c0, J[h], code[h]) ? 1u : 0u;
-                        } else {
-                            for (int q = 0; q < n; ++q)
-                                if (box_gap2(s_lo[q], s_hi[q], jl[h], jh[h]) < rcm2 &&
-                                    (other || keep_in_group(c0 + q, J[h], code[h])))
-                                    cm |= 1u << q;
-                        }
+                        for (int q = 0; q < n; ++q)
+                            if (box_gap2(s_lo[q], s_hi[q], jl[h], jh[h]) < rcm2 &&
+                                (other || keep_in_group(c0 + q, J[h], code[h])))
+                                cm |= 1u << q;
                     }
                     if (cm) {
                         const bool self = !other && code[h] == 0u && ((cm >> (J[h] - c0)) & 1u);
@@ -886,47 +877,11 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
                         if (fl && slot < 0) slot = A.pool_base + pb + __popc(ob & lt);
                     }
                     const bool ok = fl && slot < A.mask_cap;
-                    if (A.group == 1) {
-                        // warp-cooperative: for each flagged lane L, every lane
-                        // tests its partner entries against L's cluster and the
-                        // bits are OR-reduced over the warp
-                        for (unsigned f = fb; f; f &= f - 1u) {
-                            const int L = __ffs(f) - 1;
-                            const int JL = __shfl_sync(FULL, J[h], L);
-                            unsigned e0 = 0u, e1 = 0u, s0 = 0u, s1 = 0u;
-#pragma unroll
-                            for (int r = 0; r < kPartnerBatch; ++r) {
-                                const int v = pk[r];
-                                if (v >= 0 && (v >> 7) == JL) {
-                                    const int bit = v & 63;
-                                    const unsigned m = 1u << (bit & 31);
-                                    if (v & 64) {
-                                        if (bit < 32) s0 |= m;
-                                        else s1 |= m;
-                                    } else {
-                                        if (bit < 32) e0 |= m;
-                                        else e1 |= m;
-                                    }
-                                }
-                            }
-                            e0 = __reduce_or_sync(FULL, e0);
-                            e1 = __reduce_or_sync(FULL, e1);
-                            s0 = __reduce_or_sync(FULL, s0);
-                            s1 = __reduce_or_sync(FULL, s1);
-                            if (lane == L && ok) {
-                                unsigned long long ex = ((unsigned long long)e1 << 32) | e0;
-                                if (code[h] == 0u && J[h] == c0) ex |= kSelfTriangle;
-                                A.gmask[slot] = make_ulonglong2(ex, ((unsigned long long)s1 << 32) | s0);
-                            }
-                        }
-                    }
                     if (fl) {
                         if (ok) {
                             ulonglong2 *rec = A.gmask + slot * A.group;
-                            if (A.group != 1)
-                                entry_masks(s_pslot, s_link, hs >= 0 ? s_head[hs] : kLinkEnd, c0, cm, J[h], code[h],
-                                            rec);
-                            if (all_flag && A.group != 1) {  // the table overflowed: scan every partner
+                            entry_masks(s_pslot, s_link, hs >= 0 ? s_head[hs] : kLinkEnd, c0, cm, J[h], code[h], rec);
+                            if (all_flag) {  // the table overflowed: scan every partner
                                 for (unsigned ccm = cm; ccm; ccm &= ccm - 1u) {
                                     const int q2 = __ffs(ccm) - 1;
                                     ulonglong2 r = rec[q2];
@@ -945,6 +900,279 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
                         } else {
                             atomicOr(A.status, ST_CAPACITY);
                             ent.x &= ~kExclFlag;
+                        }
+                    }
+                }
+                // entry r (in scan order) to segment r % kListSegs, position r / kListSegs
+                const unsigned bh = __ballot_sync(FULL, hit);
+                if (hit) {
+                    const int r = ntot + __popc(bh & lt);
+                    const int q = r / kListSegs;
+                    if (q < seg_cap) LA[(long long)(r % kListSegs) * seg_cap + q] = ent;
+                }
+                ntot += __popc(bh);
+            }
+        }
+        __syncwarp();  // the owner table and column lists are rewritten by the next round
+    }
+    if (lane < kListSegs) {
+        const int m = (ntot + kListSegs - 1 - lane) / kListSegs;
+        A.glist_n[(long long)g * kListSegs + lane] = min(m, seg_cap);
+        if (m > seg_cap) atomicOr(A.status, ST_CAPACITY);
+    }
+}
+
+// A4 for groups of one cluster (the default tile shape): the lists and masks
+// of k_glist with group = 1, entry for entry, by a kernel that uses what one
+// cluster allows.
+//
+// * Half of the candidates are never looked at.  keep_groups keeps J > g when
+//   the indices differ in parity and J < g when they share it, and the
+//   clusters of another column all lie on one side of g: its window is
+//   walked with stride 2 from the first index of the right parity.  (Windows
+//   of the own column, and windows across a z image, where the parity of J
+//   can jump, are walked with stride 1 and tested.)
+// * No hash table: a group's partner clusters set bits of a 1,024-bit map
+//   (index modulo 1,024); a hit whose bit is set gets its masks built by the
+//   whole warp from the partner entries (one to four per lane, in registers),
+//   and is flagged when they are not empty (or the tile is the self tile).
+//
+// Bound by the instructions of each warp's dependent chain: at 23,500 atoms
+// the groups are one wave of 20 warps per SM.  Against k_glist for the same
+// lists: rebuild + forces 85.6 -> 83.0 us at 23,500 atoms, 48.6 -> 46.2 us at
+// 6,144, 2129 -> 1988 us at 999,999.  64 registers (8 blocks per SM): 72 cost
+// 22 us at 999,999 atoms, 56 gain 6 us there and cost 1 us at 23,500.
+constexpr int kGList1MinBlocks = 8;
+constexpr int kMapWords = 32;  // partner-cluster map: 1,024 bits
+
+__global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(GListArgs A)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = blockIdx.x * kGListWarps + w;  // the group is cluster g
+    __shared__ unsigned s_map_all[kGListWarps][kMapWords];
+    __shared__ int s_col_all[kGListWarps][32];
+    __shared__ int4 s_ci_all[kGListWarps][32];    // per window: jb, nj, first virtual index - stride offset, code | stride 2
+    __shared__ float2 s_co_all[kGListWarps][32];  // per window: x, y image shift
+    __shared__ unsigned char s_own_all[kGListWarps][kOwnCap];
+    unsigned *s_map = s_map_all[w];
+    s_map[lane] = 0u;
+    pdl_entry();
+    if (g >= A.counts[4]) return;  // the whole warp
+    const unsigned lt = (1u << lane) - 1u;
+    int *s_col = s_col_all[w];
+    int4 *s_ci = s_ci_all[w];
+    float2 *s_co = s_co_all[w];
+    unsigned char *s_own = s_own_all[w];
+    const int K = A.K, np = kCluster * K;  // partner entries, at most 128
+    const float inv_K = 1.0f / (float)K;
+    // the partners of the group's atoms: three dependent loads, every round's
+    // in flight together (partner cluster << 7 | is14 << 6 | bit 8 a + jj)
+    int pk[kPartnerBatch];
+#pragma unroll
+    for (int r = 0; r < kPartnerBatch; ++r) {
+        const int t = r * 32 + lane;
+        int rr;
+        pk[r] = t < np ? A.perm[g * kCluster + div_small(t, K, inv_K, rr)] : -1;
+    }
+    const float4 lo = A.bb[2 * g], hi = A.bb[2 * g + 1];
+    const SysDesc &S = A.sys[A.clus_sys[g]];
+#pragma unroll
+    for (int r = 0; r < kPartnerBatch; ++r) {
+        int rr;
+        div_small(r * 32 + lane, K, inv_K, rr);
+        pk[r] = pk[r] >= 0 ? A.part_orig[(long long)pk[r] * K + rr] : -1;
+    }
+#pragma unroll
+    for (int r = 0; r < kPartnerBatch; ++r) {
+        if (pk[r] >= 0) {
+            const int v = A.inv[pk[r] >> 1];
+            int rr;
+            const int a = div_small(r * 32 + lane, K, inv_K, rr);
+            const int pc = v / kCluster;
+            pk[r] = (pc << 7) | ((pk[r] & 1) << 6) | (a * kCluster + (v & (kCluster - 1)));
+            atomicOr(&s_map[(pc >> 5) & (kMapWords - 1)], 1u << (pc & 31));
+        }
+    }
+    __syncwarp();
+    const float rcm = A.rcm, rcm2 = rcm * rcm;
+    const int cxa = max(-S.nx, (int)floorf((lo.x - rcm) * S.inv_w[0]));
+    const int cxb = min(2 * S.nx - 1, (int)floorf((hi.x + rcm) * S.inv_w[0]));
+    const int cya = max(-S.ny, (int)floorf((lo.y - rcm) * S.inv_w[1]));
+    const int cyb = min(2 * S.ny - 1, (int)floorf((hi.y + rcm) * S.inv_w[1]));
+    const float Lz = S.L[2];
+    // conservative margin of the column-geometry test (binning rounds in FP32)
+    const float cmarg = 1e-3f + 1e-6f * fmaxf(S.L[0], S.L[1]);
+    const int ncx = cxb - cxa + 1, ncand = ncx * (cyb - cya + 1);
+    const int seg_cap = A.cap / kListSegs;
+    uint2 *LA = A.glist + (long long)g * A.cap;
+    int ntot = 0;  // entries so far (entry r goes to segment r % kListSegs)
+    const long long loc_base = (long long)g * kMaskRecsPerCluster;  // the group's own mask records
+    int nloc = 0;
+    const float inv_ncx = 1.0f / (float)ncx;
+    for (int c_lo = 0; c_lo < ncand; c_lo += 32) {
+        // the candidate columns of this round whose geometry (a lower bound
+        // of the xy gap) passes, compacted in order
+        const int cc = c_lo + lane;
+        bool pass = false;
+        int ccx = 0, ccy = 0;
+        if (cc < ncand) {
+            ccy = div_small(cc, ncx, inv_ncx, ccx);
+            const int cy = cya + ccy, cx = cxa + ccx;
+            const float gcx = fmaxf(fmaxf(cx * S.w[0] - hi.x, lo.x - (cx + 1) * S.w[0]) - cmarg, 0.0f);
+            const float gcy = fmaxf(fmaxf(cy * S.w[1] - hi.y, lo.y - (cy + 1) * S.w[1]) - cmarg, 0.0f);
+            pass = gcx * gcx + gcy * gcy < rcm2;
+        }
+        const unsigned b = __ballot_sync(FULL, pass);
+        if (pass) s_col[__popc(b & lt)] = ccx | (ccy << 16);
+        const int npass = __popc(b);
+        __syncwarp();
+        if (npass == 0) continue;
+        const int c = lane < npass ? s_col[lane] : -1;
+        int jb = 0, nj = 0, va = 0, cnt = 0, stride = 1;
+        uint32_t code_xy = 0u;
+        float ox = 0.0f, oy = 0.0f;
+        if (c >= 0) {
+            const int cy = cya + (c >> 16), cx = cxa + (c & 0xFFFF);
+            const int ky = cy < 0 ? cy + S.ny : (cy >= S.ny ? cy - S.ny : cy);
+            const int kx = cx < 0 ? cx + S.nx : (cx >= S.nx ? cx - S.nx : cx);
+            const uint32_t sy = cy < 0 ? 1u : (cy >= S.ny ? 2u : 0u);
+            const uint32_t sx = cx < 0 ? 1u : (cx >= S.nx ? 2u : 0u);
+            ox = sx == 1u ? -S.L[0] : (sx == 2u ? S.L[0] : 0.0f);
+            oy = sy == 1u ? -S.L[1] : (sy == 2u ? S.L[1] : 0.0f);
+            code_xy = sx | (sy << 2);
+            const int col = S.col_begin + ky * S.nx + kx;
+            jb = A.col_slot[col] / kCluster;
+            nj = A.col_slot[col + 1] / kCluster - jb;
+            // z window over the virtual indices v (image -L: v - nj, 0: v, +L: v + nj)
+            // from the column's z-bin index, one bin wider on each side
+            // than the FP32 bin arithmetic needs
+            const int2 *zt = A.zbin + S.zb_begin + (long long)(col - S.col_begin) * (S.nzb + 1);
+            const float za = lo.z - rcm, zb = hi.z + rcm;
+            const int ba = (int)floorf((za < 0.0f ? za + Lz : za) * S.inv_dz) - 1;
+            const int bz = (int)floorf((zb >= Lz ? zb - Lz : zb) * S.inv_dz) + 1;
+            const int vlo = zt[min(max(ba, 0), S.nzb)].x - (za < 0.0f ? nj : 0);
+            const int vhi = zt[min(max(bz, 0), S.nzb)].y + (zb >= Lz ? nj : 0);  // one past
+            if (vhi > vlo) {
+                va = vlo;
+                cnt = vhi - vlo;
+                // another column, one z image: the indices of one parity only
+                const int img = vlo < 0 ? -nj : (vlo >= nj ? nj : 0);  // J = jb + v - img
+                if ((g < jb || g >= jb + nj) && vhi - img <= nj && vlo - img >= 0) {
+                    const int J0 = jb + vlo - img;
+                    const int want = (jb > g ? 1 : 0) ^ (g & 1);  // above g: other parity, below: the same
+                    const int skip = (J0 ^ want) & 1;
+                    va += skip;
+                    cnt = (cnt - skip + 1) >> 1;
+                    stride = 2;
+                }
+            }
+        }
+        // flatten the windows of the 32 lanes
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int off = incl - cnt, total = __shfl_sync(FULL, incl, 31);
+        s_ci[lane] = make_int4(jb, nj, va - stride * off, (int)code_xy | (stride << 8));
+        s_co[lane] = make_float2(ox, oy);
+        for (int t = off; t < min(off + cnt, kOwnCap); ++t) s_own[t] = (unsigned char)lane;
+        __syncwarp();
+        for (int p0 = 0; p0 < total; p0 += 64) {
+            // both rounds' candidates and box loads first
+            int J[2];
+            uint32_t code[2];
+            float4 jl[2], jh[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int p = p0 + 32 * h + lane;
+                // owner lane: the last lane whose window starts at or before p
+                int src = 0;
+                if (p0 + 32 * h + 31 < kOwnCap) {
+                    src = p < total ? s_own[p] : 0;
+                } else {
+#pragma unroll
+                    for (int step = 16; step >= 1; step >>= 1) {
+                        const int o2 = __shfl_sync(FULL, off, src + step);
+                        if (o2 <= p) src += step;
+                    }
+                }
+                J[h] = -1;
+                code[h] = 0u;
+                jl[h] = jh[h] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (p < total) {
+                    const int4 ci = s_ci[src];
+                    const float2 co = s_co[src];
+                    J[h] = window_cluster(A.bb, p * (ci.w >> 8) + ci.z, ci.x, ci.y, (uint32_t)ci.w & 0xFFu, co.x, co.y,
+                                          Lz, code[h], jl[h], jh[h]);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (p0 + 32 * h >= total) break;  // the whole warp
+                const bool self = J[h] == g && code[h] == 0u;
+                const bool hit = J[h] >= 0 && box_gap2(lo, hi, jl[h], jh[h]) < rcm2 &&
+                                 (J[h] == g ? keep_in_group(g, g, code[h]) : keep_groups(g, J[h]));
+                // entries that may hold a partner: masks by the whole warp,
+                // every lane testing its partner entries against the entry's
+                // cluster
+                const bool may = hit && (self || ((s_map[(J[h] >> 5) & (kMapWords - 1)] >> (J[h] & 31)) & 1u));
+                bool fl = self && hit;
+                unsigned long long ex = fl ? kSelfTriangle : 0ull, s14 = 0ull;
+                for (unsigned f = __ballot_sync(FULL, may); f; f &= f - 1u) {
+                    const int L = __ffs(f) - 1;
+                    const int JL = __shfl_sync(FULL, J[h], L);
+                    unsigned e0 = 0u, e1 = 0u, s0 = 0u, s1 = 0u;
+#pragma unroll
+                    for (int r = 0; r < kPartnerBatch; ++r) {
+                        if (r * 32 >= np) break;  // the whole warp
+                        const int v = pk[r];
+                        if (v >= 0 && (v >> 7) == JL) {
+                            const int bit = v & 63;
+                            const unsigned m = 1u << (bit & 31);
+                            if (v & 64) {
+                                if (bit < 32) s0 |= m;
+                                else s1 |= m;
+                            } else {
+                                if (bit < 32) e0 |= m;
+                                else e1 |= m;
+                            }
+                        }
+                    }
+                    e0 = __reduce_or_sync(FULL, e0);
+                    e1 = __reduce_or_sync(FULL, e1);
+                    s0 = __reduce_or_sync(FULL, s0);
+                    s1 = __reduce_or_sync(FULL, s1);
+                    if (lane == L) {
+                        ex |= ((unsigned long long)e1 << 32) | e0;
+                        s14 = ((unsigned long long)s1 << 32) | s0;
+                        fl = fl || (ex | s14) != 0ull;
+                    }
+                }
+                uint2 ent = make_uint2((uint32_t)J[h] | (code[h] << kShiftBit), 1u);
+                const unsigned fb = __ballot_sync(FULL, fl);
+                if (fb) {
+                    // a record per flagged entry: the group's own in scan
+                    // order, then the shared pool
+                    const int q = nloc + __popc(fb & lt);
+                    long long slot = fl && q < kMaskRecsPerCluster ? loc_base + q : -1;
+                    nloc += __popc(fb);
+                    const unsigned ob = __ballot_sync(FULL, fl && slot < 0);
+                    if (ob) {
+                        int pb = 0;
+                        if (lane == 0) pb = atomicAdd(A.pool_count, __popc(ob));
+                        pb = __shfl_sync(FULL, pb, 0);
+                        if (fl && slot < 0) slot = A.pool_base + pb + __popc(ob & lt);
+                    }
+                    if (fl) {
+                        if (slot < A.mask_cap) {
+                            A.gmask[slot] = make_ulonglong2(ex, s14);
+                            ent.x |= kExclFlag;
+                            ent.y |= (uint32_t)slot << kMaskSlotBit;
+                        } else {
+                            atomicOr(A.status, ST_CAPACITY);
                         }
                     }
                 }
@@ -1042,7 +1270,9 @@ cudaError_t launch_build_lists(nb_ctx *ctx)
     A.group = ctx->built_group;
     const size_t smem = sizeof(int) * kGListWarps * glist_warp_ints(ctx->K, ctx->built_group);
     const int64_t blocks = std::max<int64_t>(1, (ctx->grp_cap + kGListWarps - 1) / kGListWarps);
-    cudaError_t e = launch_pdl(k_glist, dim3((unsigned)blocks), dim3(kGListWarps * 32), smem, ctx->stream, A);
+    cudaError_t e = A.group == 1
+                        ? launch_pdl(k_glist1, dim3((unsigned)blocks), dim3(kGListWarps * 32), 0, ctx->stream, A)
+                        : launch_pdl(k_glist, dim3((unsigned)blocks), dim3(kGListWarps * 32), smem, ctx->stream, A);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
