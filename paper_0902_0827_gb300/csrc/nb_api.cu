@@ -310,10 +310,10 @@ nb_status nb_step(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32
     cudaError_t e = launch_build_cells(ctx, d_pos, d_q, d_type);
     const bool pme = ctx->pme != nullptr;
     if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q);
-    if (e == cudaSuccess) e = launch_build_lists(ctx);
+    if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
     if (e != cudaSuccess) return NB_ERR_CUDA;
     ctx->built = true;
-    e = launch_forces_packed(ctx, d_F, d_energy, d_virial, false, pme, pme, pme);
+    e = launch_forces_packed(ctx, d_F, d_energy, d_virial, false, pme, pme);
     return e == cudaSuccess ? NB_OK : NB_ERR_CUDA;
 }
 

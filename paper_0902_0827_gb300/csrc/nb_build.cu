@@ -945,6 +945,14 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
 constexpr int kGList1MinBlocks = 8;
 constexpr int kMapWords = 32;  // partner-cluster map: 1,024 bits
 
+// BESIDE: the PME chain, forked before this kernel, is to run beside it.  The
+// next kernel's blocks are then not let in early: the force kernel's would
+// take the registers that the PME spread needs, and hold them while they wait
+// for the lists.  (With the equal shared-memory split of launch_pdl_split:
+// rebuild + forces with PME 125.5 -> 113.3 us at 23,500 atoms, the MD step
+// 127 -> 114 us; without the second force launch that used to follow the PME
+// chain, 109 and 106 us.)
+template <bool BESIDE>
 __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(GListArgs A)
 {
     const unsigned FULL = 0xffffffffu;
@@ -957,7 +965,8 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
     __shared__ unsigned char s_own_all[kGListWarps][kOwnCap];
     unsigned *s_map = s_map_all[w];
     s_map[lane] = 0u;
-    pdl_entry();
+    pdl_wait();
+    if (!BESIDE) pdl_trigger();
     if (g >= A.counts[4]) return;  // the whole warp
     const unsigned lt = (1u << lane) - 1u;
     int *s_col = s_col_all[w];
@@ -1225,12 +1234,12 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
     // the column counts are zero here: zeroed at create and by the scan of
     // the previous build's binning kernel, which leaves a copy for the sort
     const int tb = 256;
-    cudaError_t e = launch_pdl(k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, d.sys, d.atom_sys, d.wpos, d.atom_col,
+    cudaError_t e = launch_pdl_split(ctx->pme, k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, d.sys, d.atom_sys, d.wpos, d.atom_col,
                    d.col_count, ctx->n_cols, ctx->n_sys, d.col_slot, d.stage_fix, ctx->col_cap, d.counts, d.status,
                    ctx->group, d.col_grp,
                    host_in ? AtomPack{d_q, d_type, ctx->pp.n_types, d.atom_t} : AtomPack{nullptr, nullptr, 0, nullptr});
     if (e == cudaSuccess)
-        e = launch_pdl(!d_q ? k_colsort<kPackNone> : (host_in ? k_colsort<kPackAtomT> : k_colsort<kPackGather>),
+        e = launch_pdl_split(ctx->pme, !d_q ? k_colsort<kPackNone> : (host_in ? k_colsort<kPackAtomT> : k_colsort<kPackGather>),
                        dim3(ctx->n_cols), dim3(kSortThreads), 0, st, (const int *)d.col_count + ctx->n_cols + 1,
                        d.col_slot, d.col_sys, d.sys, (const int *)d.stage_fix, ctx->col_cap, d.stage,
                        (const int *)d.atom_col, d.wpos, d.xyzq, d.tslot, d.perm, d.inv, d.bb, d.clus_sys, d.zbin,
@@ -1242,7 +1251,7 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
     return cudaGetLastError();
 }
 
-cudaError_t launch_build_lists(nb_ctx *ctx)
+cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme)
 {
     auto &d = ctx->d;
     GListArgs A;
@@ -1271,7 +1280,8 @@ cudaError_t launch_build_lists(nb_ctx *ctx)
     const size_t smem = sizeof(int) * kGListWarps * glist_warp_ints(ctx->K, ctx->built_group);
     const int64_t blocks = std::max<int64_t>(1, (ctx->grp_cap + kGListWarps - 1) / kGListWarps);
     cudaError_t e = A.group == 1
-                        ? launch_pdl(k_glist1, dim3((unsigned)blocks), dim3(kGListWarps * 32), 0, ctx->stream, A)
+                        ? launch_pdl_split(beside_pme, beside_pme ? k_glist1<true> : k_glist1<false>, dim3((unsigned)blocks),
+                                     dim3(kGListWarps * 32), 0, ctx->stream, A)
                         : launch_pdl(k_glist, dim3((unsigned)blocks), dim3(kGListWarps * 32), smem, ctx->stream, A);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

@@ -359,31 +359,23 @@ __device__ __forceinline__ long long tile_fixed(float f, bool &ovf)
     return __float2ll_rn((ok ? f : 0.0f) * 4294967296.0f);
 }
 
-// Work units are taken without a claim first: warp w of block b of the main
-// launch starts with unit b + w gridDim (so that few units spread over all
-// SMs), and every further unit is claimed from the counter, which counts from
-// the n_first units of the first round.  A helper launch (min_left > 0; its
-// warps have no first unit) claims from the start, but only while at least
-// min_left units are left (the launch's own warps finish the rest sooner than
-// a late helper unit would).  A warp claims its next unit when the current
-// one's entries are done, so that the counter's latency hides behind the
-// unit's sums: a claim made before the unit ran kept a unit from the idle
-// warps for a whole unit's time (13 us at 23,500 atoms), and with fewer units
-// than warps some warps ran two units and others none.
-__device__ __forceinline__ int claim_unit(const ForceArgs &A, int n_first, int n_units, int min_left)
-{
-    if (min_left > 0 && n_units - n_first - *(volatile const int *)A.work < min_left) return n_units;
-    return n_first + atomicAdd(A.work, 1);
-}
+// Work units are taken without a claim first: warp w of block b starts with
+// unit b + w gridDim (so that few units spread over all SMs), and every further
+// unit is claimed from the counter, which counts from the n_first units of the
+// first round.  A warp claims its next unit when the current one's entries
+// are done, so that the counter's latency hides behind the unit's sums: a
+// claim made before the unit ran kept a unit from the idle warps for a whole
+// unit's time (13 us at 23,500 atoms), and with fewer units than warps some
+// warps ran two units and others none.
+__device__ __forceinline__ int claim_unit(const ForceArgs &A, int n_first) { return n_first + atomicAdd(A.work, 1); }
 
 // (Taken on lane 0 and broadcast like a claim: with the index computed on every
 // lane the compiler treats it as uniform and the entry loop comes out 12 %
 // slower.)
-__device__ __forceinline__ int first_unit(const ForceArgs &A, int n_first, int n_units, int min_left, int w)
+__device__ __forceinline__ int first_unit(int w)
 {
     int u = 0;
-    if ((threadIdx.x & 31) == 0)
-        u = min_left == 0 ? (int)blockIdx.x + w * (int)gridDim.x : claim_unit(A, n_first, n_units, min_left);
+    if ((threadIdx.x & 31) == 0) u = (int)blockIdx.x + w * (int)gridDim.x;
     return __shfl_sync(kFull, u, 0);
 }
 
@@ -575,7 +567,7 @@ __host__ __device__ inline size_t tile_warp_bytes(int G)
 }
 
 template <int G, int RAD, bool VIRIAL, bool DEBUG>
-__global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_force(ForceArgs A, int parts, int n_first, int min_left)
+__global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_force(ForceArgs A, int parts, int n_first)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_val[kTileWarps][kTaskVals];
@@ -604,7 +596,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
     float wimg[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // image virial of the current unit
     long long wv = 0;  // lane k < 6: fixed-point image virial component k of the current system
     bool ovf = false;  // a force sum out of the fixed-point range
-    int u = first_unit(A, n_first, n_units, min_left, w);
+    int u = first_unit(w);
     while (u < n_units) {
         const Unit U = unit_of(A, u, parts);
         int u_next = 0;
@@ -703,7 +695,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                 }
                 __syncwarp();  // the staging buffer is rewritten by the next batch
             }
-            if (lane == 0) u_next = claim_unit(A, n_first, n_units, min_left);
+            if (lane == 0) u_next = claim_unit(A, n_first);
             // force on the group's atoms: each lane's partials summed over the
             // 4 lanes of the same atom (jb) in FP32 (a fixed butterfly: every
             // lane ends with the same bits), then lane jb adds clusters c with
@@ -734,7 +726,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
             }
             __syncwarp();  // the i atoms and partials are rewritten by the next unit
         } else if (lane == 0) {
-            u_next = claim_unit(A, n_first, n_units, min_left);
+            u_next = claim_unit(A, n_first);
         }
         u = __shfl_sync(kFull, u_next, 0);
     }
@@ -974,7 +966,7 @@ __host__ __device__ inline size_t tile1_warp_bytes() { return (size_t)kBatch1 * 
 
 template <int W, int RAD, bool VIRIAL, bool DEBUG>
 __global__ void __launch_bounds__(W * 32, ACENB_TILE_MIN_BLOCKS * kTileWarps / W) k_force1(ForceArgs A, int parts,
-                                                                                        int n_first, int min_left)
+                                                                                        int n_first)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_val[W][kTaskVals];
@@ -998,7 +990,7 @@ __global__ void __launch_bounds__(W * 32, ACENB_TILE_MIN_BLOCKS * kTileWarps / W
     float wimg[3] = {0.0f, 0.0f, 0.0f};
     long long wv = 0;
     bool ovf = false;
-    int u = first_unit(A, n_first, n_units, min_left, w);
+    int u = first_unit(w);
     while (u < n_units) {
         const Unit U = unit_of(A, u, parts);
         // what needs only the unit's group and segment is loaded before the
@@ -1071,7 +1063,7 @@ __global__ void __launch_bounds__(W * 32, ACENB_TILE_MIN_BLOCKS * kTileWarps / W
                 }
                 __syncwarp();  // the staging buffer is rewritten by the next batch
             }
-            if (lane == 0) u_next = claim_unit(A, n_first, n_units, min_left);
+            if (lane == 0) u_next = claim_unit(A, n_first);
             // force on the i atoms: the 8 lanes of each atom summed in FP32
             // (a fixed butterfly), then lanes jj < 3 add atom ih, jj = 3..5
             // atom ih + 4 in fixed point
@@ -1102,7 +1094,7 @@ __global__ void __launch_bounds__(W * 32, ACENB_TILE_MIN_BLOCKS * kTileWarps / W
                 ovf = false;
             }
         } else if (lane == 0) {
-            u_next = claim_unit(A, n_first, n_units, min_left);
+            u_next = claim_unit(A, n_first);
         }
         u = __shfl_sync(kFull, u_next, 0);
     }
@@ -1261,7 +1253,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint(ForceArgs A, int par
     int cur_sys = -1;
     float Lx = 0.0f, Ly = 0.0f, Lz = 0.0f, gE_lj = 0.0f, gE_c = 0.0f;
     bool ovf = false;
-    int u = first_unit(A, n_first, n_units, 0, w);
+    int u = first_unit(w);
     while (u < n_units) {
         int u_next = 0;
         const Unit U = unit_of(A, u, parts);
@@ -1319,7 +1311,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint(ForceArgs A, int par
                 }
                 __syncwarp();  // the staging buffers are rewritten by the next batch
             }
-            if (lane == 0) u_next = claim_unit(A, n_first, n_units, 0);
+            if (lane == 0) u_next = claim_unit(A, n_first);
             // i-side terms: the 4 lanes of each atom summed in FP32 (fixed
             // butterfly), then lane jb adds clusters c with c % 4 == jb
 #pragma unroll
@@ -1348,7 +1340,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint(ForceArgs A, int par
             }
             __syncwarp();
         } else if (lane == 0) {
-            u_next = claim_unit(A, n_first, n_units, 0);
+            u_next = claim_unit(A, n_first);
         }
         u = __shfl_sync(kFull, u_next, 0);
     }
@@ -1488,7 +1480,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint1(ForceArgs A, int pa
     int cur_sys = -1;
     float Lx = 0.0f, Ly = 0.0f, Lz = 0.0f, gE_lj = 0.0f, gE_c = 0.0f;
     bool ovf = false;
-    int u = first_unit(A, n_first, n_units, 0, w);
+    int u = first_unit(w);
     while (u < n_units) {
         int u_next = 0;
         const Unit U = unit_of(A, u, parts);
@@ -1532,7 +1524,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint1(ForceArgs A, int pa
                 }
                 __syncwarp();  // the staging buffers are rewritten by the next batch
             }
-            if (lane == 0) u_next = claim_unit(A, n_first, n_units, 0);
+            if (lane == 0) u_next = claim_unit(A, n_first);
             // i-side terms: the 8 lanes of each atom summed in FP32 (a fixed
             // butterfly), then lanes jj < 4 add component jj of atom ih and
             // lanes jj >= 4 component jj - 4 of atom ih + 4
@@ -1554,7 +1546,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint1(ForceArgs A, int pa
                 ovf = false;
             }
         } else if (lane == 0) {
-            u_next = claim_unit(A, n_first, n_units, 0);
+            u_next = claim_unit(A, n_first);
         }
         u = __shfl_sync(kFull, u_next, 0);
     }
@@ -1802,13 +1794,13 @@ size_t tile_smem_bytes(int T, int G) { return lj_table_bytes(T) + (size_t)kTileW
 
 // beside_pme: the PME chain, forked before the list kernel, runs on its side
 // stream during this kernel; the persistent grid then leaves one block slot
-// per SM free, so that the PME kernels run alongside instead of after it,
-// and a second launch of the same kernel, one block per SM on the side
-// stream behind the PME chain (and the lists), takes units from the same
-// counter once the chain is done (helper).  Which block takes which unit
-// does not change any result.
+// (of kTileWarps warps) per SM free, so that the PME kernels run alongside
+// instead of after it.  Which block takes which unit does not change any
+// result.  (A second launch behind the PME chain that took units from the same
+// counter made up for a chain that started late; now that the chain starts
+// with the lists it costs 4 us of the PME step and 7 us of an MD step.)
 template <int G, int RAD, bool VIRIAL, bool DEBUG>
-static void launch_force_g(nb_ctx *ctx, const ForceArgs &A, bool beside_pme, bool helper)
+static void launch_force_g(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     const size_t smem = tile_smem_bytes(A.P.n_types, G);
     static std::atomic<unsigned long long> optin{0};
@@ -1816,15 +1808,11 @@ static void launch_force_g(nb_ctx *ctx, const ForceArgs &A, bool beside_pme, boo
     // persistent grid: never more blocks than can be resident at once
     int resident = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_force<G, RAD, VIRIAL, DEBUG>, kTileWarps * 32, smem);
-    const int per_sm = helper ? 1 : std::max(1, std::min(ctx->tune.blocks_per_sm, resident) - (beside_pme ? 1 : 0));
+    const int per_sm = std::max(1, std::min(ctx->tune.blocks_per_sm, resident) - (beside_pme ? 1 : 0));
     const int parts = ctx->tune.list_split > 0 ? ctx->tune.list_split : kDefaultListSplit;
-    // the main launch's warps take the first units; a helper claims units
-    // while more are left than the main launch has warps
-    const int n_first = helper ? ctx->num_sms * std::max(1, std::min(ctx->tune.blocks_per_sm, resident) - 1) * kTileWarps
-                               : ctx->num_sms * per_sm * kTileWarps;
-    const int min_left = helper ? n_first : 0;
-    launch_pdl(k_force<G, RAD, VIRIAL, DEBUG>, dim3(ctx->num_sms * per_sm), dim3(kTileWarps * 32), smem,
-               helper ? pme_side_stream(ctx) : ctx->stream, A, parts, n_first, min_left);
+    const int blocks = ctx->num_sms * per_sm;
+    launch_pdl(k_force<G, RAD, VIRIAL, DEBUG>, dim3(blocks), dim3(kTileWarps * 32), smem, ctx->stream, A, parts,
+               blocks * kTileWarps);
 }
 
 // Blocks of W warps of k_force1 that an SM holds (-1: not asked yet; the
@@ -1842,18 +1830,15 @@ static int force1_resident(nb_ctx *ctx, size_t smem)
 }
 
 template <int W, int RAD, bool VIRIAL, bool DEBUG>
-static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, int resident, size_t smem, bool beside_pme, bool helper)
+static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, int resident, size_t smem, bool beside_pme)
 {
     constexpr int per = kTileWarps / W;  // blocks of W warps in the tuning's unit of kTileWarps warps
-    const int all = std::min(ctx->tune.blocks_per_sm * per, resident);
-    const int main_per_sm = std::max(1, all - (beside_pme ? per : 0));
-    const int per_sm = helper ? per : main_per_sm;
+    // beside PME 8 of the 24 warps' room is left: 109.4 us a step at 23,500
+    // atoms (4: 110.2, 12: 116, none: 121)
+    const int per_sm = std::max(1, std::min(ctx->tune.blocks_per_sm * per, resident) - (beside_pme ? per : 0));
     const int parts = ctx->tune.list_split > 0 ? ctx->tune.list_split : kDefaultListSplit;
-    // the main launch's warps take the first units; a helper claims units
-    // while more are left than the main launch has warps
-    const int n_first = ctx->num_sms * main_per_sm * W;
-    launch_pdl(k_force1<W, RAD, VIRIAL, DEBUG>, dim3(ctx->num_sms * per_sm), dim3(W * 32), smem,
-               helper ? pme_side_stream(ctx) : ctx->stream, A, parts, n_first, helper ? n_first : 0);
+    const int blocks = ctx->num_sms * per_sm;
+    launch_pdl(k_force1<W, RAD, VIRIAL, DEBUG>, dim3(blocks), dim3(W * 32), smem, ctx->stream, A, parts, blocks * W);
 }
 
 // Blocks of 4 warps: they start and end in smaller steps than blocks of 8
@@ -1863,29 +1848,22 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, int resident, size_
 // with many types (above about 26) an SM holds fewer warps in blocks of 4
 // than in blocks of 8, and blocks of 8 are taken.
 template <int RAD, bool VIRIAL, bool DEBUG>
-static void launch_force_1(nb_ctx *ctx, const ForceArgs &A, bool beside_pme, bool helper)
+static void launch_force_1(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     const size_t table = lj_table_bytes(A.P.n_types);
     const size_t smem4 = table + 4 * tile1_warp_bytes(), smem8 = table + 8 * tile1_warp_bytes();
     const int r4 = force1_resident<4, RAD, VIRIAL, DEBUG>(ctx, smem4);
     const int r8 = force1_resident<8, RAD, VIRIAL, DEBUG>(ctx, smem8);
-    if (r4 >= 2 * r8) launch_force_1w<4, RAD, VIRIAL, DEBUG>(ctx, A, r4, smem4, beside_pme, helper);
-    else launch_force_1w<8, RAD, VIRIAL, DEBUG>(ctx, A, r8, smem8, beside_pme, helper);
+    if (r4 >= 2 * r8) launch_force_1w<4, RAD, VIRIAL, DEBUG>(ctx, A, r4, smem4, beside_pme);
+    else launch_force_1w<8, RAD, VIRIAL, DEBUG>(ctx, A, r8, smem8, beside_pme);
 }
 
 template <int RAD, bool VIRIAL, bool DEBUG>
-static void launch_force_t(nb_ctx *ctx, const ForceArgs &A, bool beside_pme, bool helper)
+static void launch_force_t(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
-    helper = helper && beside_pme;
-    // the lists are the last work on the context's stream here: the side
-    // stream waits for them before the helper
-    if (helper && pme_side_after_lists(ctx) != cudaSuccess) return;
-    for (int h = 0; h < (helper ? 2 : 1); ++h) {  // h = 1: the helper behind the PME chain
-        if (ctx->built_group == 1) launch_force_1<RAD, VIRIAL, DEBUG>(ctx, A, beside_pme, h == 1);
-        else if (ctx->built_group == 4) launch_force_g<4, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme, h == 1);
-        else launch_force_g<8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme, h == 1);
-        if (h == 1) pme_side_rejoin(ctx);
-    }
+    if (ctx->built_group == 1) launch_force_1<RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+    else if (ctx->built_group == 4) launch_force_g<4, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+    else launch_force_g<8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
 }
 
 // The packed constants of a parameter block.
@@ -1981,7 +1959,7 @@ cudaError_t launch_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, con
 }
 
 cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, double *d_virial, bool debug_pairs,
-                                 bool pme, bool beside_pme, bool helper)
+                                 bool pme, bool beside_pme)
 {
     auto &d = ctx->d;
     ForceArgs A = make_args(ctx);
@@ -1991,17 +1969,17 @@ cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, doub
     const bool prof = ctx->profiling && ctx->prof_n < (int)ctx->prof_ev.size() / 2;
     if (prof) cudaEventRecord(ctx->prof_ev[2 * ctx->prof_n], ctx->stream);
     if (debug_pairs) {  // the pair set does not depend on the radial functions
-        if (ewald) launch_force_t<1, false, true>(ctx, A, beside_pme, helper);
-        else launch_force_t<0, false, true>(ctx, A, beside_pme, helper);
+        if (ewald) launch_force_t<1, false, true>(ctx, A, beside_pme);
+        else launch_force_t<0, false, true>(ctx, A, beside_pme);
     } else if (ctx->tab_n > 0) {
-        if (virial) launch_force_t<2, true, false>(ctx, A, beside_pme, helper);
-        else launch_force_t<2, false, false>(ctx, A, beside_pme, helper);
+        if (virial) launch_force_t<2, true, false>(ctx, A, beside_pme);
+        else launch_force_t<2, false, false>(ctx, A, beside_pme);
     } else if (ewald) {
-        if (virial) launch_force_t<1, true, false>(ctx, A, beside_pme, helper);
-        else launch_force_t<1, false, false>(ctx, A, beside_pme, helper);
+        if (virial) launch_force_t<1, true, false>(ctx, A, beside_pme);
+        else launch_force_t<1, false, false>(ctx, A, beside_pme);
     } else {
-        if (virial) launch_force_t<0, true, false>(ctx, A, beside_pme, helper);
-        else launch_force_t<0, false, false>(ctx, A, beside_pme, helper);
+        if (virial) launch_force_t<0, true, false>(ctx, A, beside_pme);
+        else launch_force_t<0, false, false>(ctx, A, beside_pme);
     }
     if (prof) {
         cudaEventRecord(ctx->prof_ev[2 * ctx->prof_n + 1], ctx->stream);
@@ -2020,10 +1998,10 @@ cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, doub
         const long long *pf = pme ? pme_forces_acc(ctx) : nullptr, *ps = pme ? pme_sums_acc(ctx) : nullptr;
         const double pself = pme ? pme_self_coef(ctx) : 0.0;
         if (virial)
-            launch_pdl(k_unpack_forces<true>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc, d_F,
+            launch_pdl_split(ctx->pme, k_unpack_forces<true>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc, d_F,
                        d.xyzq, d.atom_sys, d.sys_acc, ctx->n_sys, en, vi, pf, ps, pself);
         else
-            launch_pdl(k_unpack_forces<false>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc,
+            launch_pdl_split(ctx->pme, k_unpack_forces<false>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc,
                        d_F, d.xyzq, d.atom_sys, d.sys_acc, ctx->n_sys, en, vi, pf, ps, pself);
     }
     return cudaGetLastError();

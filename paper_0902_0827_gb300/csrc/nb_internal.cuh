@@ -246,28 +246,42 @@ __device__ __forceinline__ float fixed_to_float(long long v)
 // a plain launch), then launch_dependents lets the next kernel's blocks be
 // scheduled while this one runs, so consecutive launches do not leave the
 // GPU idle.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_entry()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_trigger();
 }
 
-// Launch with programmatic stream serialization (see pdl_entry).
+// Launch with programmatic stream serialization (see pdl_entry).  shared:
+// with the largest shared-memory carve-out.  An SM changes its split between
+// L1 and shared memory only when it is empty, so kernels that are to share
+// SMs with the force kernel, which needs most of it, have to run with the same
+// split (the steps with PME, where two chains run side by side).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                       Args &&...args)
+cudaError_t launch_pdl_split(bool shared, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = shared ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+{
+    return launch_pdl_split(false, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // i-group slots for a context: every column's clusters form groups of
@@ -293,17 +307,15 @@ cudaError_t launch_build(nb_ctx *ctx, const float *d_pos);
 // then the cluster-pair lists
 cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q = nullptr,
                                const int32_t *d_type = nullptr);
-cudaError_t launch_build_lists(nb_ctx *ctx);
+// beside_pme: the PME chain was forked before and is to run beside the lists
+cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme = false);
 cudaError_t launch_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type,
                           float *d_F, double *d_energy, double *d_virial, bool debug_pairs);
 // launch_forces after its pack (and, when pme_forked, the PME fork): the
 // short-range kernel, the PME join and the unpack; beside_pme: the PME chain
-// was forked early enough to share the SMs with the short-range kernel;
-// helper: a second launch of the short-range kernel behind the PME chain
-// takes units from the same counter (worth it when the PME chain ends well
-// before the short-range kernel)
+// was forked early enough to share the SMs with the short-range kernel
 cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, double *d_virial, bool debug_pairs,
-                                 bool pme_forked, bool beside_pme, bool helper = false);
+                                 bool pme_forked, bool beside_pme);
 size_t force_smem_for(int T, int scap, int K);
 cudaError_t launch_pack(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type, bool zero_sums);
 cudaError_t launch_type_grad(nb_ctx *ctx, const double *gsig_tab, const double *geps_tab, double *gsig, double *geps);
@@ -315,11 +327,6 @@ cudaError_t launch_pme(nb_ctx *ctx, const float *d_pos, const float *d_q);
 // sums: also the pair-correction energy and virial (the forces always)
 // side_first: launched on the side stream before the PME chain (work that
 // is independent of the short-range path, e.g. the MD step's bonded terms).
-// The PME side stream; after_lists makes it wait for the pair lists (an event
-// on the context's stream), rejoin moves the join event to its current end.
-cudaStream_t pme_side_stream(const nb_ctx *ctx);
-cudaError_t pme_side_after_lists(nb_ctx *ctx);
-cudaError_t pme_side_rejoin(nb_ctx *ctx);
 cudaError_t launch_pme_fork(nb_ctx *ctx, const float *d_pos, const float *d_q, bool sums = true,
                             cudaError_t (*side_first)(nb_ctx *, cudaStream_t, const float *) = nullptr);
 cudaError_t launch_pme_join(nb_ctx *ctx);

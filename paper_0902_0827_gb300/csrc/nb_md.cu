@@ -791,7 +791,7 @@ static cudaError_t launch_bonded(nb_ctx *ctx, cudaStream_t st, const float *d_po
     const int terms = M.nb + M.na + M.nd;
     if (terms == 0) return cudaSuccess;
     const int blocks = std::max(1, std::min((terms + 255) / 256, 4 * ctx->num_sms));
-    return launch_pdl(k_md_bonded, dim3(blocks), dim3(256), 0, st, M.nb, M.na, M.nd,
+    return launch_pdl_split(ctx->pme, k_md_bonded, dim3(blocks), dim3(256), 0, st, M.nb, M.na, M.nd,
                       (const int2 *)M.bonds, (const float2 *)M.bond_p, (const int4 *)M.angles,
                       (const float2 *)M.angle_p, (const int4 *)M.dihedrals, (const float4 *)M.dihedral_p, d_pos,
                       box_of(ctx), M.bacc, M.acc);
@@ -801,9 +801,8 @@ static cudaError_t launch_bonded(nb_ctx *ctx, cudaStream_t st, const float *d_po
 // bonded terms.  The PME chain needs the sorted atoms but not the pair
 // lists, so it is forked onto its side stream right after the column sort
 // and the charge pack: it overlaps the list kernel and the short-range
-// kernel, and behind it a helper launch of the short-range kernel takes
-// units from the same counter; the bonded terms (positions only) run on a
-// stream of their own, off both.  sums: the energies of this evaluation are
+// kernel; the bonded terms (positions only) run on a stream of their own,
+// off both.  sums: the energies of this evaluation are
 // reported (the PME pair-correction energies are summed only then).
 static cudaError_t md_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type, bool sums,
                              bool unpack = true)
@@ -819,10 +818,10 @@ static cudaError_t md_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, 
         if (e == cudaSuccess) e = cudaEventRecord(M.bjoin, M.bside);
     }
     if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, sums);
-    if (e == cudaSuccess) e = launch_build_lists(ctx);
+    if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
     if (e != cudaSuccess) return e;
     ctx->built = true;
-    e = launch_forces_packed(ctx, unpack ? M.Fnb : nullptr, unpack ? M.enb : nullptr, nullptr, false, pme, pme, pme);
+    e = launch_forces_packed(ctx, unpack ? M.Fnb : nullptr, unpack ? M.enb : nullptr, nullptr, false, pme, pme);
     if (e != cudaSuccess) return e;
     if (pme) return bside ? cudaStreamWaitEvent(ctx->stream, M.bjoin, 0) : cudaSuccess;
     return launch_bonded(ctx, ctx->stream, d_pos);
@@ -997,14 +996,14 @@ extern "C" nb_status nb_md_step(nb_ctx *ctx, float *d_pos, float *d_vel, const f
         M.have_forces = true;
     }
     for (int s = 0; s < n_steps && e == cudaSuccess; ++s) {
-        e = launch_pdl(k_md_first, dim3(ib), dim3(64), 0, st, M.n_free, M.nw, P,
+        e = launch_pdl_split(ctx->pme, k_md_first, dim3(ib), dim3(64), 0, st, M.n_free, M.nw, P,
                        (const unsigned long long *)M.step, (const int *)M.free_atoms, (const int4 *)M.waters,
                        (const float *)M.mass, (const float *)M.sigv, (const float *)M.Ftot, d_pos, d_vel, B, M.acc,
                        ctx->d.status);
         // the second half reads the short-range sums itself (no unpack kernel)
         if (e == cudaSuccess) e = md_forces(ctx, d_pos, d_q, d_type, d_energy && s == n_steps - 1, false);
         if (e == cudaSuccess)
-            e = launch_pdl(k_md_second, dim3(ib), dim3(64), 0, st, M.n_free, M.nw, P,
+            e = launch_pdl_split(ctx->pme, k_md_second, dim3(ib), dim3(64), 0, st, M.n_free, M.nw, P,
                            M.step, (const int *)M.free_atoms, (const int4 *)M.waters,
                            (const float *)M.mass, (const float *)M.sigv,
                            NbSums{ctx->d.inv, ctx->d.facc, ctx->pme ? pme_forces_acc(ctx) : nullptr}, M.bacc,

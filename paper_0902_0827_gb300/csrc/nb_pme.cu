@@ -123,7 +123,6 @@ struct PmeState {
     // context's stream, so it overlaps the short-range kernel
     cudaStream_t side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
-    cudaEvent_t lists = nullptr;  // the pair lists are built (the short-range helper may start)
     PmeGeom g{};
     PmeCorr c{};
 };
@@ -668,7 +667,6 @@ void pme_free(nb_ctx *ctx)
     }
     if (p->fork) cudaEventDestroy(p->fork);
     if (p->join) cudaEventDestroy(p->join);
-    if (p->lists) cudaEventDestroy(p->lists);
     void *ptrs[] = {p->grid, p->fq, p->gfac, p->pacc, p->acc};
     for (void *q : ptrs)
         if (q) cudaFree(q);
@@ -688,7 +686,7 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     auto &d = ctx->d;
     const dim3 sgrid(g.K1, (g.K2 + g.Ty - 1) / g.Ty);
     const size_t smem = 2 * sizeof(int) * g.Ty * g.K3;
-    cudaError_t e = launch_pdl(k_pme_spread<N>, sgrid, dim3(kPmeThreads), smem, st, g, (const SysDesc *)d.sys,
+    cudaError_t e = launch_pdl_split(true, k_pme_spread<N>, sgrid, dim3(kPmeThreads), smem, st, g, (const SysDesc *)d.sys,
                                (const int *)d.col_slot, (const float4 *)d.xyzq, (const int *)d.perm, d_q, P.grid, P.acc);
     if (e != cudaSuccess) return e;
     if (cufftSetStream(P.fwd, st) != CUFFT_SUCCESS || cufftExecR2C(P.fwd, P.grid, (cufftComplex *)P.fq) != CUFFT_SUCCESS)
@@ -697,7 +695,7 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     const float a = ctx->pp.alpha;
     const float pi2_over_a2 = (float)(M_PI * M_PI / ((double)a * (double)a));
     const int sb = std::max(1, std::min((half + 255) / 256, 2 * ctx->num_sms));
-    e = launch_pdl(k_pme_solve, dim3(sb), dim3(256), 0, st, half, g, pi2_over_a2, (const float *)P.gfac, P.fq, P.acc);
+    e = launch_pdl_split(true, k_pme_solve, dim3(sb), dim3(256), 0, st, half, g, pi2_over_a2, (const float *)P.gfac, P.fq, P.acc);
     if (e != cudaSuccess) return e;
     if (cufftSetStream(P.inv, st) != CUFFT_SUCCESS || cufftExecC2R(P.inv, (cufftComplex *)P.fq, P.grid) != CUFFT_SUCCESS)
         return cudaErrorUnknown;
@@ -705,7 +703,7 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     const int S = (int)ctx->slot_cap;
     const int gt = 256;
     const int gb = std::max(1, std::min((S * G + gt - 1) / gt, 16 * ctx->num_sms));
-    return launch_pdl(k_pme_gather<N>, dim3(gb), dim3(gt), 0, st, g, P.c, S, (const int *)d.counts,
+    return launch_pdl_split(true, k_pme_gather<N>, dim3(gb), dim3(gt), 0, st, g, P.c, S, (const int *)d.counts,
                       (const int *)d.perm, (const int *)d.inv, (const float4 *)d.xyzq, d_pos, d_q,
                       (const float *)P.grid, (const int *)d.part_orig, ctx->K, sums ? 1 : 0, P.pacc, P.acc, d.status);
 }
@@ -736,17 +734,6 @@ cudaError_t launch_pme_fork(nb_ctx *ctx, const float *d_pos, const float *d_q, b
     if (e == cudaSuccess) e = cudaEventRecord(P.join, P.side);
     return e;
 }
-
-cudaStream_t pme_side_stream(const nb_ctx *ctx) { return ctx->pme->side; }
-
-cudaError_t pme_side_after_lists(nb_ctx *ctx)
-{
-    PmeState &P = *ctx->pme;
-    cudaError_t e = cudaEventRecord(P.lists, ctx->stream);
-    return e == cudaSuccess ? cudaStreamWaitEvent(P.side, P.lists, 0) : e;
-}
-
-cudaError_t pme_side_rejoin(nb_ctx *ctx) { return cudaEventRecord(ctx->pme->join, ctx->pme->side); }
 
 cudaError_t launch_pme_join(nb_ctx *ctx)
 {
@@ -831,10 +818,9 @@ extern "C" nb_status nb_set_pme(nb_ctx *ctx, const nb_pme_params *p)
     if (e == cudaSuccess) e = cudaMalloc(&P->pacc, sizeof(long long) * 3 * std::max<int64_t>(ctx->slot_cap, 1));
     if (e == cudaSuccess) e = cudaMalloc(&P->acc, sizeof(long long) * kPmeAcc);
     if (e == cudaSuccess) e = cudaMemset(P->acc, 0, sizeof(long long) * kPmeAcc);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->lists, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         pme_free(ctx);
         return e == cudaErrorMemoryAllocation ? NB_ERR_OOM : NB_ERR_CUDA;
