@@ -38,14 +38,13 @@ __device__ __forceinline__ int warp_aggregated_add(int *counter_base, int key)
     return base + __popc(peers & ((1u << lane) - 1u));
 }
 
-// Block-wide exclusive scan of the padded column sizes (one block).  Fills
-// the column slot offsets, the totals and the per-system slot/cluster
-// ranges; then the first i-group of every column (ceil(clusters / group)
+// Block-wide exclusive scan of the padded column sizes (one block; systems of
+// many columns, see kDirectCols).  Fills the column slot offsets and the
+// totals; then the first i-group of every column (ceil(clusters / group)
 // groups per column), copying each column's count behind the histogram for
 // the column sort and zeroing the histogram for the next build.
-__device__ void scan_columns(int n_cols, int n_sys, int *__restrict__ col_count, int *__restrict__ col_slot,
-                             SysDesc *__restrict__ sys, int *__restrict__ counts, int group,
-                             int *__restrict__ col_grp)
+__device__ void scan_columns(int n_cols, int *__restrict__ col_count, int *__restrict__ col_slot,
+                             int *__restrict__ counts, int group, int *__restrict__ col_grp)
 {
     __shared__ int warp_sum[32];
     __shared__ int carry;
@@ -106,12 +105,6 @@ __device__ void scan_columns(int n_cols, int n_sys, int *__restrict__ col_count,
     }
     __syncthreads();
     }
-    for (int s = threadIdx.x; s < n_sys; s += blockDim.x) {
-        int c0 = sys[s].col_begin, c1 = c0 + sys[s].nx * sys[s].ny;
-        sys[s].slot_begin = col_slot[c0];
-        sys[s].clus_begin = col_slot[c0] / kCluster;
-        sys[s].clus_end = col_slot[c1] / kCluster;
-    }
 }
 
 // The step's charges and types when they are in host memory, read by the
@@ -131,14 +124,14 @@ struct AtomPack {
 // (warp-aggregated atomics, whose returned counts are the atoms' places in
 // their column): each atom goes to its place in its column's fixed-capacity
 // staging row (stage_fix[col * col_cap + place]; a place at or beyond
-// col_cap is left to the column sort's fallback).  The last block to finish
-// scans the histogram.  col_count[n_cols] is the completion ticket (zero on
-// entry, reset on exit).
-__global__ void k_bin(int n, const float *__restrict__ pos, SysDesc *__restrict__ sys,
+// col_cap is left to the column sort's fallback).  With scan, the last block
+// to finish scans the histogram; col_count[n_cols] is then the completion
+// ticket (zero on entry, reset on exit).
+__global__ void k_bin(int n, const float *__restrict__ pos, const SysDesc *__restrict__ sys,
                       const int *__restrict__ atom_sys, float4 *__restrict__ wpos, int *__restrict__ atom_col,
                       int *__restrict__ col_count, int n_cols, int n_sys, int *__restrict__ col_slot,
                       int *__restrict__ stage_fix, int col_cap, int *__restrict__ counts, int *__restrict__ status,
-                      int group, int *__restrict__ col_grp, AtomPack ap)
+                      int group, int *__restrict__ col_grp, int scan, AtomPack ap)
 {
     pdl_entry();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
@@ -175,6 +168,7 @@ __global__ void k_bin(int n, const float *__restrict__ pos, SysDesc *__restrict_
     }
     const int place = warp_aggregated_add(col_count, col);
     if (col >= 0 && place < col_cap) stage_fix[(long long)col * col_cap + place] = a;
+    if (!scan) return;  // the column sort sums the counts itself
     // last block: the histogram is complete.  The barrier orders the block's
     // counter updates before thread 0's fence, which (cumulatively) orders
     // them before the ticket.
@@ -187,7 +181,7 @@ __global__ void k_bin(int n, const float *__restrict__ pos, SysDesc *__restrict_
     __syncthreads();
     if (!last) return;
     __threadfence();
-    scan_columns(n_cols, n_sys, col_count, col_slot, sys, counts, group, col_grp);
+    scan_columns(n_cols, col_count, col_slot, counts, group, col_grp);
     if (threadIdx.x == 0) col_count[n_cols] = 0;
 }
 
@@ -234,6 +228,15 @@ __device__ void bitonic_sort(unsigned long long *skey, int P)
     }
 }
 
+// Up to this many columns (a system or batch) every block of the column sort
+// sums the counts of the columns before its own (a few loads per thread, in
+// flight with its other first loads) and the list kernel zeroes the
+// histogram; above, the last block of the binning kernel scans the histogram
+// once (the blocks' loads grow with the square of the columns).  Rebuild +
+// forces with the scan and without: 82.5 and 79.9 us at 23,500 atoms (196
+// columns), 45.4 and 43.0 us at 6,144, 933 and 914 us for 64 boxes (4,508
+// columns), 1991 and 1977 us at 999,999 (2,401).
+constexpr int kDirectCols = 8192;
 constexpr int kRankSortMax = 256;  // columns up to this many atoms are rank-sorted (no barriers)
 
 // Per-atom inputs of the force kernels packed by the column sort when the
@@ -296,20 +299,41 @@ __device__ __forceinline__ int sorted_type(const ColPack &pk, int t)
 // (94 for the gathering instance) in both the step and the MD step.
 template <int PACK>
 __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
-    const int *__restrict__ col_count, const int *__restrict__ col_slot, const int *__restrict__ col_sys,
-    const SysDesc *__restrict__ sys, const int *__restrict__ stage_fix, int col_cap, int *__restrict__ stage,
+    const int *__restrict__ col_count, int *__restrict__ col_slot, int direct, int *__restrict__ counts,
+    const int *__restrict__ col_sys, const SysDesc *__restrict__ sys, const int *__restrict__ stage_fix, int col_cap, int *__restrict__ stage,
     const int *__restrict__ atom_col, const float4 *__restrict__ wpos,
     float4 *__restrict__ xyzq, int *__restrict__ tslot, int *__restrict__ perm, int *__restrict__ inv,
     float4 *__restrict__ bb, int *__restrict__ clus_sys, int2 *__restrict__ zbin, int group,
-    const int *__restrict__ col_grp, int2 *__restrict__ grp, int *__restrict__ clus_grp, ColPack pk)
+    int *__restrict__ col_grp, int2 *__restrict__ grp, int *__restrict__ clus_grp, ColPack pk)
 {
     pdl_entry();
     __shared__ unsigned long long skey[kSortSmem];
     __shared__ float4 sp[kSortSmem];
+    __shared__ int s_pre[2][kSortThreads / 32];
     const int c = blockIdx.x;
     const int tid = threadIdx.x;
     const int n = col_count[c];
-    const int base = col_slot[c];
+    if (direct) {  // clusters and i-groups of the columns before this one
+        int ncl = 0, ngr = 0;
+        for (int k = tid; k < c; k += kSortThreads) {
+            const int q = (col_count[k] + kCluster - 1) / kCluster;
+            ncl += q;
+            ngr += group == 1 ? q : (q + group - 1) / group;
+        }
+        ncl = __reduce_add_sync(0xffffffffu, ncl);
+        ngr = __reduce_add_sync(0xffffffffu, ngr);
+        if ((tid & 31) == 0) {
+            s_pre[0][tid >> 5] = ncl;
+            s_pre[1][tid >> 5] = ngr;
+        }
+    }
+    // (after the next barrier)
+    auto first_slot = [&]() {
+        int v = 0;
+        for (int k = 0; k < kSortThreads / 32; ++k) v += s_pre[0][k];
+        return direct ? v * kCluster : col_slot[c];
+    };
+    int base = 0;
     const int npad = (n + kCluster - 1) / kCluster * kCluster;
     // the column's atoms: its staging row, or, when the column outgrew the
     // row's capacity (strongly uneven density), gathered here from the
@@ -319,6 +343,7 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
         __shared__ int s_fill;
         if (tid == 0) s_fill = 0;
         __syncthreads();
+        base = first_slot();
         const SysDesc &S0 = sys[col_sys[c]];
         for (int a = S0.atom_begin + tid; a < S0.atom_begin + S0.n_atoms; a += blockDim.x)
             if (atom_col[a] == c) stage[base + atomicAdd(&s_fill, 1)] = a;
@@ -338,6 +363,7 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
             skey[k] = key;
         }
         __syncthreads();
+        base = first_slot();
         bitonic_sort(skey, P);
         for (int k = tid; k < n; k += blockDim.x) {
             const int a = (int)(unsigned)(skey[k] & 0xffffffffull);
@@ -371,6 +397,7 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
             }
         }
         __syncthreads();
+        base = first_slot();
         if (nper <= 1) rank_keys<1>(skey, n, key, rank);
         else if (nper <= 2) rank_keys<2>(skey, n, key, rank);
         else if (nper <= 4) rank_keys<4>(skey, n, key, rank);
@@ -389,6 +416,8 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
             }
         }
     } else {
+        __syncthreads();
+        base = first_slot();
         for (int k = tid; k < n; k += blockDim.x) {
             const int a = src[k];
             float4 pa = wpos[a];
@@ -421,6 +450,25 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
     __syncthreads();
     // cluster bounding boxes over the real atoms of each 8-slot cluster
     const int nclus = npad / kCluster;
+    int grp0 = 0;  // the column's first i-group
+    if (direct) {
+        for (int k = 0; k < kSortThreads / 32; ++k) grp0 += s_pre[1][k];
+        if (tid == 0) {  // what the scan writes otherwise
+            const int ngr = group == 1 ? nclus : (nclus + group - 1) / group;
+            col_slot[c] = base;
+            col_grp[c] = grp0;
+            if (c == 0) counts[5] = 0;
+            if (c == (int)gridDim.x - 1) {
+                col_slot[c + 1] = base + npad;
+                col_grp[c + 1] = grp0 + ngr;
+                counts[0] = base + npad;
+                counts[1] = (base + npad) / kCluster;
+                counts[4] = grp0 + ngr;
+            }
+        }
+    } else {
+        grp0 = col_grp[c];
+    }
     for (int q = tid; q < nclus; q += blockDim.x) {
         float lx = INFINITY, ly = INFINITY, lz = INFINITY, hx = -INFINITY, hy = -INFINITY, hz = -INFINITY;
         for (int k = q * kCluster; k < min(n, (q + 1) * kCluster); ++k) {
@@ -435,7 +483,7 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
         // i-groups: runs of `group` consecutive clusters of the column
         // (groups of one are numbered like their clusters: no table)
         if (group != 1) {
-            const int gi = col_grp[c] + q / group;
+            const int gi = grp0 + q / group;
             clus_grp[I] = gi;
             if (q % group == 0) grp[gi] = make_int2(I, min(group, nclus - q));
         }
@@ -644,7 +692,15 @@ struct GListArgs {
     float rcm;
     int cap;                 // entries per group (all segments)
     int group;               // clusters per group of the lists being built (records hold `group` mask pairs)
+    int *col_count;          // the column histogram, zeroed here for the next build
+    int n_zero;              // its columns (0: zeroed by the binning kernel's scan)
 };
+
+__device__ __forceinline__ void zero_histogram(const GListArgs &A)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < A.n_zero) A.col_count[t] = 0;
+}
 
 constexpr int kGListWarps = 4;  // groups (warps) per block of the list kernel
 #ifndef ACENB_GLIST_MIN_BLOCKS
@@ -666,6 +722,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
         s_head_all[w][t] = kLinkEnd;
     }
     pdl_entry();
+    zero_histogram(A);
     if (g >= A.counts[4]) return;  // the whole warp
     const unsigned lt = (1u << lane) - 1u;
     const int2 gr = A.grp[g];
@@ -967,6 +1024,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
     s_map[lane] = 0u;
     pdl_wait();
     if (!BESIDE) pdl_trigger();
+    zero_histogram(A);
     if (g >= A.counts[4]) return;  // the whole warp
     const unsigned lt = (1u << lane) - 1u;
     int *s_col = s_col_all[w];
@@ -1231,17 +1289,19 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
     cudaStream_t st = ctx->stream;
     const int N = (int)ctx->n_atoms;
     const bool host_in = d_q && inputs_in_host_memory(ctx, d_q);
-    // the column counts are zero here: zeroed at create and by the scan of
-    // the previous build's binning kernel, which leaves a copy for the sort
+    // the column counts are zero here: zeroed at create and by the previous
+    // build (its list kernel, or the scan of its binning kernel, which leaves
+    // a copy for the sort)
+    const int direct = ctx->n_cols <= kDirectCols ? 1 : 0;
     const int tb = 256;
     cudaError_t e = launch_pdl_split(ctx->pme, k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, d.sys, d.atom_sys, d.wpos, d.atom_col,
                    d.col_count, ctx->n_cols, ctx->n_sys, d.col_slot, d.stage_fix, ctx->col_cap, d.counts, d.status,
-                   ctx->group, d.col_grp,
+                   ctx->group, d.col_grp, 1 - direct,
                    host_in ? AtomPack{d_q, d_type, ctx->pp.n_types, d.atom_t} : AtomPack{nullptr, nullptr, 0, nullptr});
     if (e == cudaSuccess)
         e = launch_pdl_split(ctx->pme, !d_q ? k_colsort<kPackNone> : (host_in ? k_colsort<kPackAtomT> : k_colsort<kPackGather>),
-                       dim3(ctx->n_cols), dim3(kSortThreads), 0, st, (const int *)d.col_count + ctx->n_cols + 1,
-                       d.col_slot, d.col_sys, d.sys, (const int *)d.stage_fix, ctx->col_cap, d.stage,
+                       dim3(ctx->n_cols), dim3(kSortThreads), 0, st, (const int *)d.col_count + (direct ? 0 : ctx->n_cols + 1),
+                       d.col_slot, direct, d.counts, d.col_sys, d.sys, (const int *)d.stage_fix, ctx->col_cap, d.stage,
                        (const int *)d.atom_col, d.wpos, d.xyzq, d.tslot, d.perm, d.inv, d.bb, d.clus_sys, d.zbin,
                        ctx->group, d.col_grp, d.grp, d.clus_grp,
                        ColPack{d_q, d_type, ctx->pp.n_types, d.atom_t, d.facc, d.sys_acc, kTaskVals * ctx->n_sys,
@@ -1277,6 +1337,8 @@ cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme)
     A.rcm = ctx->pp.rc + ctx->pp.list_margin;
     A.cap = ctx->list_cap;
     A.group = ctx->built_group;
+    A.col_count = d.col_count;
+    A.n_zero = ctx->n_cols <= kDirectCols ? ctx->n_cols : 0;
     const size_t smem = sizeof(int) * kGListWarps * glist_warp_ints(ctx->K, ctx->built_group);
     const int64_t blocks = std::max<int64_t>(1, (ctx->grp_cap + kGListWarps - 1) / kGListWarps);
     cudaError_t e = A.group == 1

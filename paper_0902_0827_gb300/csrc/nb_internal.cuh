@@ -55,8 +55,7 @@ enum : int {
     ST_TIMEOUT = 1 << 5,
 };
 
-// Per-system descriptor (device resident).  Fields marked [build] are
-// written by the binning kernels at every build.
+// Per-system descriptor (device resident).
 struct SysDesc {
     float L[3];          // box edges
     float half[3];       // 0.5 * L (FP32, exact)
@@ -66,9 +65,6 @@ struct SysDesc {
     int atom_begin;      // first atom in the concatenated input arrays
     int n_atoms;
     int col_begin;       // first global column
-    int slot_begin;      // [build] first sorted slot
-    int clus_begin;      // [build] first cluster
-    int clus_end;        // [build] one past the last cluster
     // z-bin index of every column: bins of height dz = Lz / nzb; per column
     // nzb + 1 pairs (first cluster with z_hi >= b dz, first cluster with
     // z_lo > (b + 1) dz), at zb_begin + local column * (nzb + 1)
@@ -128,8 +124,9 @@ struct DevBuffers {
     int *atom_t = nullptr;           // [N] range-checked types in caller order (nb_step and MD steps)
     int *part_orig = nullptr;        // [N*K] partner (orig << 1) | is14, -1 pad (static)
     int *col_sys = nullptr;          // [C] system of each column (static)
-    int *col_count = nullptr;        // [2C+1] column histogram (zero between builds); [C] = completion ticket
-                                     // of the binning kernel; [C+1+c] = column c's count for the column sort
+    int *col_count = nullptr;        // [2C+1] column histogram (zero between builds); with a scan (many columns)
+                                     // [C] = completion ticket of the binning kernel, [C+1+c] = column c's count
+                                     // for the column sort
     int *col_slot = nullptr;         // [C+1] padded slot offsets
     int *stage = nullptr;            // [S] unsorted atoms of a column whose staging row overflowed
     int *stage_fix = nullptr;        // [C * col_cap] unsorted atoms per column, fixed capacity

@@ -9,6 +9,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+import oracle
 from paper_0902_0827_gb300 import nb
 from paper_0902_0827_gb300 import systems as S
 
@@ -39,6 +40,8 @@ CASES = {
     "one_column": lambda: [_lj(57, (30.0, 30.0, 30.0), 4)],
     "droplet": lambda: [_droplets(1500, 50.0, 5)],
     "batch": lambda: [_lj(n, (18.0, 19.0, 20.0), 7 + n) for n in (9, 130, 77, 401, 8, 250)],
+    # above 8,192 columns: the binning kernel's scan instead of the column sort's own sums
+    "many_columns": lambda: [_lj(107000, (1200.0, 1200.0, 18.5), 8)],
     "waters": lambda: [S.water_box(n_waters=n) for n in (199, 307, 512)],
 }
 
@@ -59,3 +62,7 @@ def test_groups_of_one_and_four(name):
     assert np.array_equal(got[1][0], got[4][0])
     F1, F4 = got[1][1], got[4][1]
     assert np.linalg.norm(F1 - F4) <= 5e-6 * np.linalg.norm(F4)
+    if name == "many_columns":
+        Fo, _, _, n_pairs = oracle.forces(systems[0], method="cells")
+        assert n_pairs == len(got[1][0])
+        assert np.linalg.norm(F1 - Fo) <= 5e-6 * np.linalg.norm(Fo)
