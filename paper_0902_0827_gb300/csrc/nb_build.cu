@@ -12,31 +12,10 @@
 
 #include <algorithm>
 
+#include "nb_bin.cuh"
 #include "nb_internal.cuh"
 
 namespace acenb {
-
-__device__ __forceinline__ int column_of(float x, float inv_w, int n)
-{
-    int c = (int)floorf(__fmul_rn(x, inv_w));
-    if (c > n - 1) c = n - 1;
-    if (c < 0) c = 0;
-    return c;
-}
-
-// Warp-aggregated counter update: lanes with the same key (-1 = none) take
-// consecutive positions from one atomic per distinct key; returns the old
-// counter value plus the lane's rank among its peers.
-__device__ __forceinline__ int warp_aggregated_add(int *counter_base, int key)
-{
-    const unsigned peers = __match_any_sync(0xffffffffu, key);
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(peers) - 1;
-    int base = 0;
-    if (key >= 0 && lane == leader) base = atomicAdd(&counter_base[key], __popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    return base + __popc(peers & ((1u << lane) - 1u));
-}
 
 // Block-wide exclusive scan of the padded column sizes (one block; systems of
 // many columns, see kDirectCols).  Fills the column slot offsets and the
@@ -107,19 +86,6 @@ __device__ void scan_columns(int n_cols, int *__restrict__ col_count, int *__res
     }
 }
 
-// The step's charges and types when they are in host memory, read by the
-// binning kernel beside the positions (coalesced, in caller order, across
-// the host link): the charge goes to the wrapped position's w, the
-// range-checked type to atom_t, and the column sort carries both into sorted
-// order.  q = null: positions only (w = 0); device-resident charges and
-// types are gathered by the column sort instead (faster there).
-struct AtomPack {
-    const float *q;
-    const int *type;
-    int T;
-    int *atom_t;  // [N] checked types in caller order
-};
-
 // A1 + A2 + A3a: one atom per thread: wrap, column index, column histogram
 // (warp-aggregated atomics, whose returned counts are the atoms' places in
 // their column): each atom goes to its place in its column's fixed-capacity
@@ -127,47 +93,31 @@ struct AtomPack {
 // col_cap is left to the column sort's fallback).  With scan, the last block
 // to finish scans the histogram; col_count[n_cols] is then the completion
 // ticket (zero on entry, reset on exit).
-__global__ void k_bin(int n, const float *__restrict__ pos, const SysDesc *__restrict__ sys,
-                      const int *__restrict__ atom_sys, float4 *__restrict__ wpos, int *__restrict__ atom_col,
-                      int *__restrict__ col_count, int n_cols, int n_sys, int *__restrict__ col_slot,
-                      int *__restrict__ stage_fix, int col_cap, int *__restrict__ counts, int *__restrict__ status,
-                      int group, int *__restrict__ col_grp, int scan, AtomPack ap)
+__global__ void k_bin(int n, const float *__restrict__ pos, BinArgs B, const int *__restrict__ atom_sys, int n_cols,
+                      int n_sys, int *__restrict__ col_slot, int *__restrict__ counts, int group,
+                      int *__restrict__ col_grp, int scan, AtomPack ap)
 {
     pdl_entry();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    int col = -1;
+    int *col_count = B.col_count;
+    float x = 0.0f, y = 0.0f, z = 0.0f, qa = 0.0f;
+    int s = 0;
     if (a < n) {
-        const SysDesc &S = sys[n_sys == 1 ? 0 : atom_sys[a]];  // one system: no dependent load
-        float x = pos[3ll * a], y = pos[3ll * a + 1], z = pos[3ll * a + 2];
-        if (!(isfinite(x) && isfinite(y) && isfinite(z))) {
-            atomicOr(status, ST_NONFINITE);
-            x = 0.0f; y = 0.0f; z = 0.0f;
-        }
-        x = wrap_coord(x, S.L[0]);
-        y = wrap_coord(y, S.L[1]);
-        z = wrap_coord(z, S.L[2]);
-        // a finite coordinate too large for the FP32 wrap (|x| beyond ~2^24 L)
-        // is reported like a non-finite one: every later index stays in range
-        if (!(x >= 0.0f && x < S.L[0] && y >= 0.0f && y < S.L[1] && z >= 0.0f && z < S.L[2])) {
-            atomicOr(status, ST_NONFINITE);
-            x = 0.0f; y = 0.0f; z = 0.0f;
-        }
-        col = S.col_begin + column_of(y, S.inv_w[1], S.ny) * S.nx + column_of(x, S.inv_w[0], S.nx);
-        atom_col[a] = col;
-        float qa = 0.0f;
+        if (n_sys != 1) s = atom_sys[a];  // one system: no dependent load
+        x = pos[3ll * a];
+        y = pos[3ll * a + 1];
+        z = pos[3ll * a + 2];
         if (ap.q) {  // charge and checked type, read beside the position
             qa = ap.q[a];
             int t = ap.type[a];
             if (t < 0 || t >= ap.T) {
-                atomicOr(status, ST_BADTYPE);
+                atomicOr(B.status, ST_BADTYPE);
                 t = 0;
             }
             ap.atom_t[a] = t;
         }
-        wpos[a] = make_float4(x, y, z, qa);
     }
-    const int place = warp_aggregated_add(col_count, col);
-    if (col >= 0 && place < col_cap) stage_fix[(long long)col * col_cap + place] = a;
+    bin_atom(B, a < n ? a : -1, s, x, y, z, qa);
     if (!scan) return;  // the column sort sums the counts itself
     // last block: the histogram is complete.  The barrier orders the block's
     // counter updates before thread 0's fence, which (cumulatively) orders
@@ -1283,21 +1233,35 @@ static bool inputs_in_host_memory(nb_ctx *ctx, const void *p)
     return ctx->host_inputs = at.type == cudaMemoryTypeHost;
 }
 
-cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type)
+BinArgs bin_args(const nb_ctx *ctx)
+{
+    const auto &d = ctx->d;
+    return BinArgs{d.sys, d.wpos, d.atom_col, d.col_count, d.stage_fix, ctx->col_cap, d.status};
+}
+
+bool bins_elsewhere(nb_ctx *ctx, const float *d_q)
+{
+    return ctx->n_sys == 1 && ctx->n_cols <= kDirectCols && !inputs_in_host_memory(ctx, d_q);
+}
+
+cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type, bool binned)
 {
     auto &d = ctx->d;
     cudaStream_t st = ctx->stream;
     const int N = (int)ctx->n_atoms;
-    const bool host_in = d_q && inputs_in_host_memory(ctx, d_q);
+    const bool host_in = !binned && d_q && inputs_in_host_memory(ctx, d_q);
     // the column counts are zero here: zeroed at create and by the previous
     // build (its list kernel, or the scan of its binning kernel, which leaves
     // a copy for the sort)
     const int direct = ctx->n_cols <= kDirectCols ? 1 : 0;
     const int tb = 256;
-    cudaError_t e = launch_pdl_split(ctx->pme, k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, d.sys, d.atom_sys, d.wpos, d.atom_col,
-                   d.col_count, ctx->n_cols, ctx->n_sys, d.col_slot, d.stage_fix, ctx->col_cap, d.counts, d.status,
-                   ctx->group, d.col_grp, 1 - direct,
-                   host_in ? AtomPack{d_q, d_type, ctx->pp.n_types, d.atom_t} : AtomPack{nullptr, nullptr, 0, nullptr});
+    cudaError_t e = cudaSuccess;
+    if (!binned)
+        e = launch_pdl_split(ctx->pme, k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, bin_args(ctx),
+                             (const int *)d.atom_sys, ctx->n_cols, ctx->n_sys, d.col_slot, d.counts, ctx->group, d.col_grp,
+                             1 - direct,
+                             host_in ? AtomPack{d_q, d_type, ctx->pp.n_types, d.atom_t}
+                                     : AtomPack{nullptr, nullptr, 0, nullptr});
     if (e == cudaSuccess)
         e = launch_pdl_split(ctx->pme, !d_q ? k_colsort<kPackNone> : (host_in ? k_colsort<kPackAtomT> : k_colsort<kPackGather>),
                        dim3(ctx->n_cols), dim3(kSortThreads), 0, st, (const int *)d.col_count + (direct ? 0 : ctx->n_cols + 1),

@@ -116,6 +116,17 @@ struct PairConst2 {
     f32x2 exp2_c[kExp2Deg + 1];
 };
 
+// Where the binning of an atom goes (bin_atom).
+struct BinArgs {
+    const SysDesc *sys;
+    float4 *wpos;
+    int *atom_col;
+    int *col_count;
+    int *stage_fix;
+    int col_cap;
+    int *status;
+};
+
 struct DevBuffers {
     SysDesc *sys = nullptr;          // [n_sys]
     int *atom_sys = nullptr;         // [N]
@@ -302,8 +313,12 @@ inline int column_capacity(double mean_atoms) { return ((int)(2.0 * mean_atoms) 
 cudaError_t launch_build(nb_ctx *ctx, const float *d_pos);
 // the two halves of launch_build: binning, column sort and cluster boxes;
 // then the cluster-pair lists
+// binned: the atoms were binned by the kernel before (the MD half-steps, when
+// bins_elsewhere: one system, no scan, charges in device memory)
 cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q = nullptr,
-                               const int32_t *d_type = nullptr);
+                               const int32_t *d_type = nullptr, bool binned = false);
+BinArgs bin_args(const nb_ctx *ctx);
+bool bins_elsewhere(nb_ctx *ctx, const float *d_q);
 // beside_pme: the PME chain was forked before and is to run beside the lists
 cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme = false);
 cudaError_t launch_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type,

@@ -5,17 +5,20 @@
 //
 // One step of length dt from (x, v, F(x)); one lane per unconstrained atom,
 // three per rigid water (one per atom, the constraints solved on all three):
-//   k_md_first   O: v <- c v + sigma xi (c = exp(-gamma dt/2),
+//   first half   O: v <- c v + sigma xi (c = exp(-gamma dt/2),
 //                sigma = sqrt((1 - c^2) kT / m)), B: v += dt/2 F/m,
 //                A: x' = x + dt v; waters then M-SHAKE (Newton on the 3
 //                distance equations with the reference bond vectors of x):
 //                x'' = x' + disp and v += disp / dt
 //   cell list, short-range forces (+ PME), k_md_bonded
-//   k_md_second  reads the short-range (+ PME) forces from their
-//                fixed-point sums (no unpack kernel), B: v += dt/2 F/m,
+//   second half  the short-range (+ PME) forces from their fixed-point sums
+//                (no unpack kernel), B: v += dt/2 F/m,
 //                O: v <- c v + sigma xi'; waters then RATTLE
 //                (r_k . (v_a - v_b) = 0); kinetic energy; the last block
 //                writes the energies and advances the step counter
+// A call of n steps runs k_md_first, then between the evaluations
+// k_md_between (second half of a step, first half of the next and the
+// binning), and k_md_second after the last one.
 // xi: Philox4x32-10 (Salmon et al. 2011) on the counter (atom, step,
 // stream, 0) and key (seed), 24-bit uniforms, Box-Muller.  Units kcal/mol,
 // A, amu, ps: F/m in kcal/mol/A/amu times 418.4 is A/ps^2.
@@ -25,6 +28,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "nb_bin.cuh"
 #include "nb_internal.cuh"
 
 namespace acenb {
@@ -248,12 +252,11 @@ struct NbSums {
 
 __device__ __forceinline__ float3 nb_force_of(const NbSums &N, int a)
 {
-    const float sc = 2.3283064365386963e-10f;  // 2^-32
     const long long s = N.inv[a];
     const long long p0 = N.pme_f ? N.pme_f[3 * s] : 0, p1 = N.pme_f ? N.pme_f[3 * s + 1] : 0,
                     p2 = N.pme_f ? N.pme_f[3 * s + 2] : 0;
-    return make_float3(__ll2float_rn(N.facc[3 * s] + p0) * sc, __ll2float_rn(N.facc[3 * s + 1] + p1) * sc,
-                       __ll2float_rn(N.facc[3 * s + 2] + p2) * sc);
+    return make_float3(fixed_to_float(N.facc[3 * s] + p0), fixed_to_float(N.facc[3 * s + 1] + p1),
+                       fixed_to_float(N.facc[3 * s + 2] + p2));
 }
 
 // Total forces F = F_short + bonded (the fixed-point bonded sums are cleared).
@@ -282,67 +285,62 @@ __global__ void k_md_collect(int n, const float *__restrict__ Fnb, long long *__
     collect_force(a, Fnb, bacc, Ftot, fx, fy, fz);
 }
 
-// O (stream 0), B, A of atom a: returns x' = x + dt v (v updated in place).
-__device__ __forceinline__ float3 kick_drift(int a, float dt, float c, bool langevin, unsigned long long seed,
-                                             unsigned long long step, const float *__restrict__ mass,
-                                             const float *__restrict__ sigv, const float *__restrict__ Ftot,
-                                             const float *__restrict__ x, float *__restrict__ v)
+struct MdStep {
+    float dt, c;
+    bool langevin;
+    unsigned long long seed;
+    float d2oh, d2hh, tol;
+    int max_iter;
+};
+
+// O (stream 0) and B of an atom with velocity v and force f; the new position
+// is x + dt v.
+__device__ __forceinline__ float3 kick_before(float3 v, float3 f, float3 xi, float ma, float sa, const MdStep &P)
 {
-    // every load is issued first and the noise computed while they are in flight
-    float vx = v[3ll * a], vy = v[3ll * a + 1], vz = v[3ll * a + 2];
-    const float sa = langevin ? sigv[a] : 0.0f, ma = mass[a];
-    const float f0 = Ftot[3ll * a], f1 = Ftot[3ll * a + 1], f2 = Ftot[3ll * a + 2];
-    const float x0 = x[3ll * a], x1 = x[3ll * a + 1], x2 = x[3ll * a + 2];
-    if (langevin) {
-        const float3 xi = md_normals((unsigned)a, step, 0u, seed);
-        vx = fmaf(c, vx, sa * xi.x);
-        vy = fmaf(c, vy, sa * xi.y);
-        vz = fmaf(c, vz, sa * xi.z);
+    if (P.langevin) {
+        v.x = fmaf(P.c, v.x, sa * xi.x);
+        v.y = fmaf(P.c, v.y, sa * xi.y);
+        v.z = fmaf(P.c, v.z, sa * xi.z);
     }
-    const float h = 0.5f * dt * kAccel / ma;
-    vx = fmaf(h, f0, vx);
-    vy = fmaf(h, f1, vy);
-    vz = fmaf(h, f2, vz);
-    v[3ll * a] = vx;
-    v[3ll * a + 1] = vy;
-    v[3ll * a + 2] = vz;
-    return make_float3(fmaf(dt, vx, x0), fmaf(dt, vy, x1), fmaf(dt, vz, x2));
+    const float h = 0.5f * P.dt * kAccel / ma;
+    return make_float3(fmaf(h, f.x, v.x), fmaf(h, f.y, v.y), fmaf(h, f.z, v.z));
 }
 
-// B and O (stream 1) of atom a with the new forces (v updated in place).
-__device__ __forceinline__ float3 kick(int a, float dt, float c, bool langevin, unsigned long long seed,
-                                       unsigned long long step, const float *__restrict__ mass,
-                                       const float *__restrict__ sigv, const NbSums &Nb,
-                                       long long *__restrict__ bacc, float *__restrict__ Ftot, float *__restrict__ v)
+// B and O (stream 1) of an atom with the new force.
+__device__ __forceinline__ float3 kick_after(float3 v, float3 f, float3 xi, float ma, float sa, const MdStep &P)
 {
-    const float sc = 2.3283064365386963e-10f;  // 2^-32
-    // every load is issued first and the noise (integer and special-function
-    // work that needs none of them) computed while they are in flight
+    const float h = 0.5f * P.dt * kAccel / ma;
+    v = make_float3(fmaf(h, f.x, v.x), fmaf(h, f.y, v.y), fmaf(h, f.z, v.z));
+    if (P.langevin) {
+        v.x = fmaf(P.c, v.x, sa * xi.x);
+        v.y = fmaf(P.c, v.y, sa * xi.y);
+        v.z = fmaf(P.c, v.z, sa * xi.z);
+    }
+    return v;
+}
+
+__device__ __forceinline__ float3 load3(const float *__restrict__ p, int a)
+{
+    return make_float3(p[3ll * a], p[3ll * a + 1], p[3ll * a + 2]);
+}
+
+__device__ __forceinline__ void store3(float *__restrict__ p, int a, float3 v)
+{
+    p[3ll * a] = v.x;
+    p[3ll * a + 1] = v.y;
+    p[3ll * a + 2] = v.z;
+}
+
+// Total force of atom a from the sums of the last evaluation (short-range,
+// PME, bonded); the bonded sums are cleared.
+__device__ __forceinline__ float3 total_force(const NbSums &Nb, long long *__restrict__ bacc, int a)
+{
     const float3 fn = nb_force_of(Nb, a);
     const long long b0 = bacc[3ll * a], b1 = bacc[3ll * a + 1], b2 = bacc[3ll * a + 2];
-    const float ma = mass[a], sa = langevin ? sigv[a] : 0.0f;
-    const float v0 = v[3ll * a], v1 = v[3ll * a + 1], v2 = v[3ll * a + 2];
-    const float3 xi = langevin ? md_normals((unsigned)a, step, 1u, seed) : make_float3(0.0f, 0.0f, 0.0f);
-    const float fx = fn.x + __ll2float_rn(b0) * sc;
-    const float fy = fn.y + __ll2float_rn(b1) * sc;
-    const float fz = fn.z + __ll2float_rn(b2) * sc;
     bacc[3ll * a] = 0;
     bacc[3ll * a + 1] = 0;
     bacc[3ll * a + 2] = 0;
-    Ftot[3ll * a] = fx;
-    Ftot[3ll * a + 1] = fy;
-    Ftot[3ll * a + 2] = fz;
-    const float h = 0.5f * dt * kAccel / ma;
-    float vx = fmaf(h, fx, v0), vy = fmaf(h, fy, v1), vz = fmaf(h, fz, v2);
-    if (langevin) {
-        vx = fmaf(c, vx, sa * xi.x);
-        vy = fmaf(c, vy, sa * xi.y);
-        vz = fmaf(c, vz, sa * xi.z);
-    }
-    v[3ll * a] = vx;
-    v[3ll * a + 1] = vy;
-    v[3ll * a + 2] = vz;
-    return make_float3(vx, vy, vz);
+    return make_float3(fn.x + fixed_to_float(b0), fn.y + fixed_to_float(b1), fn.z + fixed_to_float(b2));
 }
 
 // Rigid water: constraint k joins (O, H1), (O, H2), (H1, H2).
@@ -373,14 +371,6 @@ __device__ __forceinline__ void solve3(const float A[3][3], const float b[3], fl
     x[1] = i10 * b[0] + i11 * b[1] + i12 * b[2];
     x[2] = i20 * b[0] + i21 * b[1] + i22 * b[2];
 }
-
-struct MdStep {
-    float dt, c;
-    bool langevin;
-    unsigned long long seed;
-    float d2oh, d2hh, tol;
-    int max_iter;
-};
 
 // M-SHAKE of one water (atoms at[], inverse masses im[]) from the reference
 // positions x to the unconstrained new positions xn: the displacements dsp
@@ -492,156 +482,217 @@ __device__ __forceinline__ float3 water_lanes3(float3 v, int base, int k)
                        __shfl_sync(0xffffffffu, v.z, base + k));
 }
 
-// First half of a step.  An unconstrained atom: O, B, A.  A water: each of
-// its three lanes kicks and drifts its atom, then M-SHAKE on the three
-// lanes: lambda by Newton iterations on |r_k''|^2 = d_k^2,
-// r_k'' = u_k + sum_l lambda_l C_kl r_l (u: new, r: reference vectors of x,
-// C_kl = s(a_k, l)/m_{a_k} - s(b_k, l)/m_{b_k}), disp_i =
-// sum_l lambda_l s(i, l) r_l / m_i, until every |g_k| / d_k^2 < tol or
-// max_iter iterations; each lane moves its atom.  New positions wrapped into
-// the box.  Block 0 clears the energy sums of this step.
-__global__ void __launch_bounds__(64) k_md_first(int n_free, int nw, MdStep P,
-                                                 const unsigned long long *__restrict__ step,
-                                                 const int *__restrict__ free_atoms, const int4 *__restrict__ waters,
-                                                 const float *__restrict__ mass, const float *__restrict__ sigv,
-                                                 const float *__restrict__ Ftot, float *__restrict__ x,
-                                                 float *__restrict__ v, Box3 B, long long *__restrict__ acc,
-                                                 int *__restrict__ status)
+// One lane's atom in the half-step kernels.
+struct MdAtom {
+    int a;                // atom, -1: none
+    float3 x, v, f;       // position, velocity, force
+    float m, s;           // mass, noise amplitude
+    float3 r[3];          // a water's bond vectors at x
+};
+
+struct MdArgs {
+    int n_free, nw;
+    MdStep P;
+    unsigned long long *step;
+    const int *free_atoms;
+    const int4 *waters;
+    const float *mass, *sigv;
+    float *Ftot, *x, *v;
+    Box3 B;
+    long long *acc;
+    int *status;
+};
+
+// The lane's atom with everything but its force loaded (all loads issued
+// before the noise is computed by the caller).
+__device__ __forceinline__ MdAtom md_load(const MdArgs &M, const MdLane &L)
 {
-    pdl_entry();
-    if (blockIdx.x == 0 && threadIdx.x < kMdAcc) acc[threadIdx.x] = 0;
-    const unsigned long long st = step[0];
-    const MdLane L = md_lane(n_free, nw);
+    MdAtom A;
+    A.a = -1;
+    A.x = A.v = A.f = make_float3(0.0f, 0.0f, 0.0f);
+    A.m = 1.0f;
+    A.s = 0.0f;
+    if (!L.active) return A;
     if (!L.water_warp) {
-        if (!L.active) return;
-        const int a = free_atoms[L.item];
-        const float3 p = kick_drift(a, P.dt, P.c, P.langevin, P.seed, st, mass, sigv, Ftot, x, v);
-        x[3ll * a] = wrap_coord(p.x, B.L[0]);
-        x[3ll * a + 1] = wrap_coord(p.y, B.L[1]);
-        x[3ll * a + 2] = wrap_coord(p.z, B.L[2]);
-        return;
+        A.a = M.free_atoms[L.item];
+    } else {
+        const int4 W = M.waters[L.item];
+        const int at[3] = {W.x, W.y, W.z};
+        A.a = L.i == 0 ? at[0] : (L.i == 1 ? at[1] : at[2]);
+        water_bonds(at, M.x, M.B, A.r);
     }
-    // water warp: every lane stays to the end (shuffles, warp barrier)
-    const int4 W = L.active ? waters[L.item] : make_int4(0, 0, 0, 0);
-    const int at[3] = {W.x, W.y, W.z};
-    const int a = L.i == 0 ? at[0] : (L.i == 1 ? at[1] : at[2]);
-    float3 r[3];  // the reference bonds (loads issued before the kick)
-    if (L.active) water_bonds(at, x, B, r);
-    float3 mine = make_float3(0.0f, 0.0f, 0.0f);
-    float im_mine = 1.0f;
-    if (L.active) {
-        mine = kick_drift(a, P.dt, P.c, P.langevin, P.seed, st, mass, sigv, Ftot, x, v);
-        im_mine = 1.0f / mass[a];
-    }
-    const int base = (threadIdx.x & 31) - L.i;
-    float3 xn[3];
-    float im[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        xn[k] = water_lanes3(mine, base, k);
-        im[k] = __shfl_sync(0xffffffffu, im_mine, base + k);
-    }
-    float3 dsp[3];
-    if (L.active && !water_shake(r, xn, im, B, P, dsp) && L.i == 0) atomicOr(status, ST_TIMEOUT);
-    __syncwarp();  // the three lanes read the reference positions x before any writes them
-    if (!L.active) return;
-    const float3 d = L.i == 0 ? dsp[0] : (L.i == 1 ? dsp[1] : dsp[2]);
-    const float idt = 1.0f / P.dt;
-    x[3ll * a] = wrap_coord(mine.x + d.x, B.L[0]);
-    x[3ll * a + 1] = wrap_coord(mine.y + d.y, B.L[1]);
-    x[3ll * a + 2] = wrap_coord(mine.z + d.z, B.L[2]);
-    v[3ll * a] = fmaf(d.x, idt, v[3ll * a]);
-    v[3ll * a + 1] = fmaf(d.y, idt, v[3ll * a + 1]);
-    v[3ll * a + 2] = fmaf(d.z, idt, v[3ll * a + 2]);
+    A.x = load3(M.x, A.a);
+    A.v = load3(M.v, A.a);
+    A.m = M.mass[A.a];
+    if (M.P.langevin) A.s = M.sigv[A.a];
+    return A;
 }
 
-// Second half of a step, same lanes: B and O with the new forces (the
-// short-range and PME forces read from their fixed-point sums); a water's
-// velocities then by RATTLE on its three lanes, mu from the 3 x 3 system
-// sum_l mu_l C_kl (r_k . r_l) = -r_k . (v_a - v_b), v_i += sum_l mu_l s(i,l) r_l / m_i;
-// kinetic energy (a water's on its first lane).  The last block to finish
-// writes the energies (short-range + long-range from their sums, the
-// fixed-point sums of acc) to energy, when given, and advances the device
-// step counter.
-__global__ void __launch_bounds__(64) k_md_second(int n_free, int nw, MdStep P,
-                                                  unsigned long long *__restrict__ step,
-                                                  const int *__restrict__ free_atoms, const int4 *__restrict__ waters,
-                                                  const float *__restrict__ mass, const float *__restrict__ sigv,
-                                                  NbSums Nb, long long *__restrict__ bacc,
-                                                  float *__restrict__ Ftot, const float *__restrict__ x,
-                                                  float *__restrict__ v, Box3 B, long long *__restrict__ acc,
-                                                  const long long *__restrict__ sys_acc, const long long *__restrict__ pme_s,
-                                                  double pme_self, double *__restrict__ energy)
+// First half of a step on the lane's atom: O, B, A; a water (its three lanes
+// with the same inputs) then M-SHAKE: lambda by Newton iterations on
+// |r_k''|^2 = d_k^2, r_k'' = u_k + sum_l lambda_l C_kl r_l (u: new, r:
+// reference vectors of x, C_kl = s(a_k, l)/m_{a_k} - s(b_k, l)/m_{b_k}),
+// disp_i = sum_l lambda_l s(i, l) r_l / m_i, until every |g_k| / d_k^2 < tol
+// or max_iter iterations; each lane moves its atom.  Writes the velocity and
+// the new position wrapped into the box, and bins the atom (bin.sys given).
+// Called by every lane of the warp.
+__device__ __forceinline__ void md_advance(const MdArgs &M, const MdLane &L, MdAtom &A, float3 xi, const BinArgs &bin)
 {
-    pdl_entry();
-    const unsigned long long st = step[0];
-    long long ke[1] = {0};
-    const MdLane L = md_lane(n_free, nw);
-    if (!L.water_warp) {
-        if (L.active) {
-            const int a = free_atoms[L.item];
-            const float3 u = kick(a, P.dt, P.c, P.langevin, P.seed, st, mass, sigv, Nb, bacc, Ftot, v);
-            ke[0] = __float2ll_rn(0.5f * mass[a] * fmaf(u.x, u.x, fmaf(u.y, u.y, u.z * u.z)) / kAccel *
-                                  4294967296.0f);
-        }
-    } else {
-        const int4 W = L.active ? waters[L.item] : make_int4(0, 0, 0, 0);
-        const int at[3] = {W.x, W.y, W.z};
-        const int a = L.i == 0 ? at[0] : (L.i == 1 ? at[1] : at[2]);
-        float3 r[3];  // the bonds (loads issued before the kick)
-        if (L.active) water_bonds(at, x, B, r);
-        float3 mine = make_float3(0.0f, 0.0f, 0.0f);
-        float m_mine = 1.0f;
-        if (L.active) {
-            mine = kick(a, P.dt, P.c, P.langevin, P.seed, st, mass, sigv, Nb, bacc, Ftot, v);
-            m_mine = mass[a];
-        }
+    const MdStep &P = M.P;
+    float3 xn = make_float3(0.0f, 0.0f, 0.0f);
+    if (A.a >= 0) {
+        A.v = kick_before(A.v, A.f, xi, A.m, A.s, P);
+        xn = make_float3(fmaf(P.dt, A.v.x, A.x.x), fmaf(P.dt, A.v.y, A.x.y), fmaf(P.dt, A.v.z, A.x.z));
+    }
+    if (L.water_warp) {
+        const float im_mine = A.a >= 0 ? 1.0f / A.m : 1.0f;
         const int base = (threadIdx.x & 31) - L.i;
-        float m[3], im[3], vv[3][3];
+        float3 xw[3], dsp[3];
+        float im[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const float3 u = water_lanes3(mine, base, k);
-            vv[k][0] = u.x;
-            vv[k][1] = u.y;
-            vv[k][2] = u.z;
-            m[k] = __shfl_sync(0xffffffffu, m_mine, base + k);
-            im[k] = 1.0f / m[k];
+            xw[k] = water_lanes3(xn, base, k);
+            im[k] = __shfl_sync(0xffffffffu, im_mine, base + k);
         }
-        if (L.active) {
-            float A[3][3], b[3], mu[3];
+        if (A.a >= 0) {
+            if (!water_shake(A.r, xw, im, M.B, P, dsp) && L.i == 0) atomicOr(M.status, ST_TIMEOUT);
+            const float3 d = L.i == 0 ? dsp[0] : (L.i == 1 ? dsp[1] : dsp[2]);
+            const float idt = 1.0f / P.dt;
+            xn = make_float3(xn.x + d.x, xn.y + d.y, xn.z + d.z);
+            A.v = make_float3(fmaf(d.x, idt, A.v.x), fmaf(d.y, idt, A.v.y), fmaf(d.z, idt, A.v.z));
+        }
+        __syncwarp();  // the three lanes read the reference positions x before any writes them
+    }
+    if (A.a >= 0) {
+        xn = make_float3(wrap_coord(xn.x, M.B.L[0]), wrap_coord(xn.y, M.B.L[1]), wrap_coord(xn.z, M.B.L[2]));
+        store3(M.x, A.a, xn);
+        store3(M.v, A.a, A.v);
+    }
+    if (bin.sys) bin_atom(bin, A.a, 0, xn.x, xn.y, xn.z, 0.0f);
+}
+
+// Second half of a step on the lane's atom: B and O with the new force; a
+// water's velocities then by RATTLE on its three lanes, mu from the 3 x 3
+// system sum_l mu_l C_kl (r_k . r_l) = -r_k . (v_a - v_b),
+// v_i += sum_l mu_l s(i,l) r_l / m_i.  Returns the kinetic energy times
+// kAccel (a water's on its first lane).
+__device__ __forceinline__ float md_finish(const MdArgs &M, const MdLane &L, MdAtom &A, float3 xi)
+{
+    if (A.a >= 0) A.v = kick_after(A.v, A.f, xi, A.m, A.s, M.P);
+    if (!L.water_warp) {
+        const float3 u = A.v;
+        return A.a >= 0 ? 0.5f * A.m * fmaf(u.x, u.x, fmaf(u.y, u.y, u.z * u.z)) : 0.0f;
+    }
+    const int base = (threadIdx.x & 31) - L.i;
+    float m[3], im[3];
+    float3 vv[3];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int ka = con_a(k), kb = con_b(k);
-                const float3 dv = make_float3(vv[ka][0] - vv[kb][0], vv[ka][1] - vv[kb][1], vv[ka][2] - vv[kb][2]);
-                b[k] = -dot3(r[k], dv);
+    for (int k = 0; k < 3; ++k) {
+        vv[k] = water_lanes3(A.v, base, k);
+        m[k] = __shfl_sync(0xffffffffu, A.m, base + k);
+        im[k] = 1.0f / m[k];
+    }
+    if (A.a < 0) return 0.0f;
+    float C[3][3], b[3], mu[3];
 #pragma unroll
-                for (int l = 0; l < 3; ++l)
-                    A[k][l] = (sgn(ka, l) * im[ka] - sgn(kb, l) * im[kb]) * dot3(r[k], r[l]);
-            }
-            solve3(A, b, mu);
-            float e = 0.0f, mx = 0.0f, my = 0.0f, mz = 0.0f;
+    for (int k = 0; k < 3; ++k) {
+        const int ka = con_a(k), kb = con_b(k);
+        const float3 dv = make_float3(vv[ka].x - vv[kb].x, vv[ka].y - vv[kb].y, vv[ka].z - vv[kb].z);
+        b[k] = -dot3(A.r[k], dv);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                float3 dv = make_float3(0.0f, 0.0f, 0.0f);
+        for (int l = 0; l < 3; ++l)
+            C[k][l] = (sgn(ka, l) * im[ka] - sgn(kb, l) * im[kb]) * dot3(A.r[k], A.r[l]);
+    }
+    solve3(C, b, mu);
+    float e = 0.0f;
 #pragma unroll
-                for (int l = 0; l < 3; ++l) dv = add3(dv, scale3(mu[l] * sgn(i, l) * im[i], r[l]));
-                const float vx = vv[i][0] + dv.x, vy = vv[i][1] + dv.y, vz = vv[i][2] + dv.z;
-                if (i == L.i) {
-                    mx = vx;
-                    my = vy;
-                    mz = vz;
-                }
-                e = fmaf(0.5f * m[i], fmaf(vx, vx, fmaf(vy, vy, vz * vz)), e);
-            }
-            v[3ll * a] = mx;
-            v[3ll * a + 1] = my;
-            v[3ll * a + 2] = mz;
-            if (L.i == 0) ke[0] = __float2ll_rn(e / kAccel * 4294967296.0f);
+    for (int i = 0; i < 3; ++i) {
+        float3 dv = make_float3(0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int l = 0; l < 3; ++l) dv = add3(dv, scale3(mu[l] * sgn(i, l) * im[i], A.r[l]));
+        const float3 u = add3(vv[i], dv);
+        if (i == L.i) A.v = u;
+        e = fmaf(0.5f * m[i], fmaf(u.x, u.x, fmaf(u.y, u.y, u.z * u.z)), e);
+    }
+    return L.i == 0 ? e : 0.0f;
+}
+
+// First half of the first step of a call (forces of the last evaluation in
+// Ftot).  Block 0 clears the energy sums of this step.
+__global__ void __launch_bounds__(64) k_md_first(MdArgs M, BinArgs bin)
+{
+    pdl_entry();
+    if (blockIdx.x == 0 && threadIdx.x < kMdAcc) M.acc[threadIdx.x] = 0;
+    const unsigned long long st = M.step[0];
+    const MdLane L = md_lane(M.n_free, M.nw);
+    MdAtom A = md_load(M, L);
+    if (A.a >= 0) A.f = load3(M.Ftot, A.a);
+    const float3 xi = M.P.langevin ? md_normals((unsigned)A.a, st, 0u, M.P.seed) : make_float3(0.0f, 0.0f, 0.0f);
+    md_advance(M, L, A, xi, bin);
+}
+
+// Between two steps of a call: the second half of one step and the first half
+// of the next on the same lanes, with the velocity, the force and a water's
+// bond vectors kept in registers, and the atoms binned for the next
+// evaluation (no energies are reported here, and the total force is not
+// stored).  One kernel for what took three (second half, first half,
+// binning), each a latency chain of its own of 4 to 5 us: ten MD steps of the
+// 23,500-atom chain with PME 1032 -> 996 us, of 2,718 atoms 765 -> 704 us.
+// The last block to finish clears the energy sums and advances the step
+// counter.
+__global__ void __launch_bounds__(64) k_md_between(MdArgs M, NbSums Nb, long long *__restrict__ bacc, BinArgs bin)
+{
+    pdl_entry();
+    const unsigned long long st = M.step[0];
+    const MdLane L = md_lane(M.n_free, M.nw);
+    MdAtom A = md_load(M, L);
+    if (A.a >= 0) A.f = total_force(Nb, bacc, A.a);
+    const float3 none = make_float3(0.0f, 0.0f, 0.0f);
+    const float3 xi1 = M.P.langevin ? md_normals((unsigned)A.a, st, 1u, M.P.seed) : none;
+    const float3 xi0 = M.P.langevin ? md_normals((unsigned)A.a, st + 1ull, 0u, M.P.seed) : none;
+    md_finish(M, L, A, xi1);
+    md_advance(M, L, A, xi0, bin);
+    __syncthreads();  // every thread has read step before the ticket
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned long long done = atomicAdd((unsigned long long *)&M.acc[kMdTicket], 1ull);
+        if (done == gridDim.x - 1ull) {
+            for (int k = 0; k < kMdAcc; ++k) M.acc[k] = 0;
+            M.step[0] = st + 1ull;
         }
     }
+}
+
+// Second half of the last step of a call (short-range and PME forces read
+// from their fixed-point sums), the total force kept for the next call;
+// kinetic energy.  The last block to finish writes the energies (short-range
+// + long-range from their sums, the fixed-point sums of acc) to energy, when
+// given, and advances the device step counter.
+__global__ void __launch_bounds__(64) k_md_second(MdArgs M, NbSums Nb, long long *__restrict__ bacc,
+                                                  const long long *__restrict__ sys_acc,
+                                                  const long long *__restrict__ pme_s, double pme_self,
+                                                  double *__restrict__ energy)
+{
+    pdl_entry();
+    const unsigned long long st = M.step[0];
+    const MdLane L = md_lane(M.n_free, M.nw);
+    MdAtom A = md_load(M, L);
+    if (A.a >= 0) A.f = total_force(Nb, bacc, A.a);
+    const float3 xi = M.P.langevin ? md_normals((unsigned)A.a, st, 1u, M.P.seed) : make_float3(0.0f, 0.0f, 0.0f);
+    const float e = md_finish(M, L, A, xi);
+    if (A.a >= 0) {
+        store3(M.Ftot, A.a, A.f);
+        store3(M.v, A.a, A.v);
+    }
+    long long *acc = M.acc;
+    long long ke[1] = {0};
     const int idx[1] = {3};
-    if (energy) md_flush<1>(ke, acc, idx);  // the kinetic energy only when reported
-    else __syncthreads();                   // (its barrier: every thread has read step before the ticket)
+    if (energy) {  // the kinetic energy only when reported
+        ke[0] = __float2ll_rn(e / kAccel * 4294967296.0f);
+        md_flush<1>(ke, acc, idx);
+    } else {
+        __syncthreads();  // every thread has read step before the ticket
+    }
     if (threadIdx.x == 0) {  // the thread that added this block's sum
         __threadfence();
         const unsigned long long done =
@@ -656,7 +707,7 @@ __global__ void __launch_bounds__(64) k_md_second(int n_free, int nw, MdStep P,
                 energy[1] = (double)e_c * (1.0 / kFixScale);
                 for (int k = 0; k < 4; ++k) energy[2 + k] = (double)va[k] * (1.0 / 4294967296.0);
             }
-            step[0] += 1ull;
+            M.step[0] += 1ull;
         }
     }
 }
@@ -805,10 +856,10 @@ static cudaError_t launch_bonded(nb_ctx *ctx, cudaStream_t st, const float *d_po
 // off both.  sums: the energies of this evaluation are
 // reported (the PME pair-correction energies are summed only then).
 static cudaError_t md_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type, bool sums,
-                             bool unpack = true)
+                             bool unpack = true, bool binned = false)
 {
     MdState &M = *ctx->md;
-    cudaError_t e = launch_build_cells(ctx, d_pos, d_q, d_type);  // q and types packed on the way
+    cudaError_t e = launch_build_cells(ctx, d_pos, d_q, d_type, binned);  // q and types packed on the way
     const bool pme = ctx->pme != nullptr;
     const bool bside = pme && M.nb + M.na + M.nd > 0;
     if (e == cudaSuccess && bside) {
@@ -995,22 +1046,24 @@ extern "C" nb_status nb_md_step(nb_ctx *ctx, float *d_pos, float *d_vel, const f
         if (e != cudaSuccess) return NB_ERR_CUDA;
         M.have_forces = true;
     }
+    const MdArgs A{M.n_free, M.nw, P, M.step, M.free_atoms, M.waters, M.mass, M.sigv, M.Ftot, d_pos, d_vel, B, M.acc,
+                   ctx->d.status};
+    const NbSums Nb{ctx->d.inv, ctx->d.facc, ctx->pme ? pme_forces_acc(ctx) : nullptr};
+    // the half-steps bin the atoms they move, where the binning needs no scan
+    const bool binned = bins_elsewhere(ctx, d_q);
+    const BinArgs bin = binned ? bin_args(ctx) : BinArgs{};
     for (int s = 0; s < n_steps && e == cudaSuccess; ++s) {
-        e = launch_pdl_split(ctx->pme, k_md_first, dim3(ib), dim3(64), 0, st, M.n_free, M.nw, P,
-                       (const unsigned long long *)M.step, (const int *)M.free_atoms, (const int4 *)M.waters,
-                       (const float *)M.mass, (const float *)M.sigv, (const float *)M.Ftot, d_pos, d_vel, B, M.acc,
-                       ctx->d.status);
-        // the second half reads the short-range sums itself (no unpack kernel)
-        if (e == cudaSuccess) e = md_forces(ctx, d_pos, d_q, d_type, d_energy && s == n_steps - 1, false);
-        if (e == cudaSuccess)
-            e = launch_pdl_split(ctx->pme, k_md_second, dim3(ib), dim3(64), 0, st, M.n_free, M.nw, P,
-                           M.step, (const int *)M.free_atoms, (const int4 *)M.waters,
-                           (const float *)M.mass, (const float *)M.sigv,
-                           NbSums{ctx->d.inv, ctx->d.facc, ctx->pme ? pme_forces_acc(ctx) : nullptr}, M.bacc,
-                           M.Ftot, (const float *)d_pos, d_vel, B, M.acc, (const long long *)ctx->d.sys_acc,
-                           ctx->pme ? pme_sums_acc(ctx) : nullptr, ctx->pme ? pme_self_coef(ctx) : 0.0,
-                           s == n_steps - 1 ? d_energy : (double *)nullptr);
+        if (s == 0)
+            e = launch_pdl_split(ctx->pme, k_md_first, dim3(ib), dim3(64), 0, st, A, bin);
+        else
+            e = launch_pdl_split(ctx->pme, k_md_between, dim3(ib), dim3(64), 0, st, A, Nb, M.bacc, bin);
+        // the half-steps read the short-range sums themselves (no unpack kernel)
+        if (e == cudaSuccess) e = md_forces(ctx, d_pos, d_q, d_type, d_energy && s == n_steps - 1, false, binned);
     }
+    if (e == cudaSuccess && n_steps > 0)
+        e = launch_pdl_split(ctx->pme, k_md_second, dim3(ib), dim3(64), 0, st, A, Nb, M.bacc,
+                             (const long long *)ctx->d.sys_acc, ctx->pme ? pme_sums_acc(ctx) : nullptr,
+                             ctx->pme ? pme_self_coef(ctx) : 0.0, d_energy);
     return e == cudaSuccess ? NB_OK : NB_ERR_CUDA;
 }
 
