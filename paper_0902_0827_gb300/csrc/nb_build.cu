@@ -1249,7 +1249,7 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
     auto &d = ctx->d;
     cudaStream_t st = ctx->stream;
     const int N = (int)ctx->n_atoms;
-    const bool host_in = !binned && d_q && inputs_in_host_memory(ctx, d_q);
+    const bool host_in = !binned && d_q && d.atom_t && inputs_in_host_memory(ctx, d_q);
     // the column counts are zero here: zeroed at create and by the previous
     // build (its list kernel, or the scan of its binning kernel, which leaves
     // a copy for the sort)

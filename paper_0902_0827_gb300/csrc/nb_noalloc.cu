@@ -20,8 +20,8 @@
 // nothing is allocated on the host heap either.
 //
 // All calls share the one array and it keeps the previous call's contents:
-// the entry point clears what must start at zero (status word, column counts,
-// energy accumulators, the sorted type array) at every call.  Calls whose
+// the entry point clears what must start at zero (status word, column counts)
+// at every call.  Calls whose
 // kernels overlap on the GPU (different streams, or several host threads at
 // once) race on the array and on the host staging buffers; callers must
 // serialise them.
@@ -52,15 +52,21 @@ constexpr long long kMaskRecs = kClus * kMaskRecsPerCluster + kClus / 2 + 64;  /
 constexpr size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Byte offsets of every scratch buffer inside the static array.
-constexpr size_t oSys = 0;
-constexpr size_t oAtomSys = oSys + a256(sizeof(SysDesc));
-constexpr size_t oAtomCol = oAtomSys + a256(4ull * kMaxAtoms);
+// What a call uploads, in one copy: the system, the type-pair table and the
+// partners, one behind the other (fitted to the system's types and partners).
+constexpr size_t kUpLj = a256(sizeof(SysDesc));
+constexpr size_t kUpBytes = kUpLj + a256(16ull * kMaxTypes * kMaxTypes) + a256(4ull * kMaxAtoms * kMaxPartners);
+constexpr size_t oUp = 0;
+// What a call clears, in one go: the status word and the column counts.
+constexpr size_t oStatus = oUp + a256(kUpBytes);
+constexpr size_t oColCount = oStatus + 16;
+constexpr size_t oAtomCol = oStatus + a256(16 + 4ull * (2 * kMaxCols + 1));
 constexpr size_t oWpos = oAtomCol + a256(4ull * kMaxAtoms);
-constexpr size_t oPart = oWpos + a256(16ull * kMaxAtoms);
-constexpr size_t oColSys = oPart + a256(4ull * kMaxAtoms * kMaxPartners);
-constexpr size_t oColCount = oColSys + a256(4ull * kMaxCols);
+// (one system: zero from the start and never written)
+constexpr size_t oAtomSys = oWpos + a256(16ull * kMaxAtoms);
+constexpr size_t oColSys = oAtomSys + a256(4ull * kMaxAtoms);
 constexpr long long kStageFix = 4 * kSlots;  // column staging rows (col_cap per column, fitted to the system)
-constexpr size_t oStageFix = oColCount + a256(4ull * (2 * kMaxCols + 1));
+constexpr size_t oStageFix = oColSys + a256(4ull * kMaxCols);
 constexpr size_t oColSlot = oStageFix + a256(4ull * kStageFix);
 constexpr size_t oStage = oColSlot + a256(4ull * (kMaxCols + 1));
 constexpr size_t oXyzq = oStage + a256(4ull * kSlots);
@@ -79,19 +85,16 @@ constexpr size_t oGlistN = oGlist + a256(8ull * kGrp * kListCap);
 constexpr size_t oGmask = oGlistN + a256(4ull * kGrp * kListSegs);
 constexpr size_t oZbin = oGmask + a256(16ull * kMaskRecs * kDefaultGroup);  // records of one-cluster groups
 constexpr size_t oCounts = oZbin + a256(8ull * kZbEntries);
-constexpr size_t oStatus = oCounts + a256(32);
-constexpr size_t oLj = oStatus + a256(16);
-constexpr size_t oDbg = oLj + a256(16ull * kMaxTypes * kMaxTypes);
+constexpr size_t oDbg = oCounts + a256(32);
 constexpr size_t kScratchBytes = oDbg + a256(16);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 // host-side staging (fixed size, no heap)
-SysDesc h_sys;
+alignas(256) unsigned char h_up[kUpBytes];
 int h_part[kMaxAtoms * kMaxPartners];
 int h_cnt[kMaxAtoms];
 double h_sg[kMaxTypes * kMaxTypes], h_ep[kMaxTypes * kMaxTypes];
-float4 h_lj[kMaxTypes * kMaxTypes];
 unsigned char *g_dev_scratch[kMaxDevices];  // cached device address per device
 
 template <class T>
@@ -145,12 +148,14 @@ extern "C" nb_status nb_forces_noalloc(const nb_params *params, const float *d_p
     if (st != NB_OK) return st;
     int K = 1;
     for (int i = 0; i < N; ++i) K = h_cnt[i] > K ? h_cnt[i] : K;
-    // repack to stride K
-    for (int i = 0; i < N; ++i)
-        for (int k = 0; k < K; ++k) h_part[i * K + k] = k < h_cnt[i] ? h_part[i * kMaxPartners + k] : -1;
     const int T = p.n_types;
-    host::make_tables(T, p.comb_rule, p.sigma, p.epsilon, p.sigma_tab, p.eps_tab, h_sg, h_ep, h_lj);
-    h_sys = S;
+    const size_t up_part = kUpLj + a256(16ull * T * T);
+    memcpy(h_up, &S, sizeof(SysDesc));
+    host::make_tables(T, p.comb_rule, p.sigma, p.epsilon, p.sigma_tab, p.eps_tab, h_sg, h_ep,
+                      reinterpret_cast<float4 *>(h_up + kUpLj));
+    int *up = reinterpret_cast<int *>(h_up + up_part);  // partners with stride K
+    for (int i = 0; i < N; ++i)
+        for (int k = 0; k < K; ++k) up[i * K + k] = k < h_cnt[i] ? h_part[i * kMaxPartners + k] : -1;
 
     // the device address of the scratch array, looked up once per device
     int dev = 0;
@@ -189,11 +194,11 @@ extern "C" nb_status nb_forces_noalloc(const nb_params *params, const float *d_p
     c.zb_total = host::zbin_entries(S);
     c.comb_rule = p.comb_rule;
     DevBuffers &d = c.d;
-    d.sys = at<SysDesc>(base, oSys);
+    d.sys = at<SysDesc>(base, oUp);
     d.atom_sys = at<int>(base, oAtomSys);
     d.atom_col = at<int>(base, oAtomCol);
     d.wpos = at<float4>(base, oWpos);
-    d.part_orig = at<int>(base, oPart);
+    d.part_orig = at<int>(base, oUp + up_part);
     d.col_sys = at<int>(base, oColSys);
     d.col_count = at<int>(base, oColCount);
     d.stage_fix = at<int>(base, oStageFix);
@@ -216,24 +221,24 @@ extern "C" nb_status nb_forces_noalloc(const nb_params *params, const float *d_p
     d.zbin = at<int2>(base, oZbin);
     d.counts = at<int>(base, oCounts);
     d.status = at<int>(base, oStatus);
-    d.lj_tab = at<float4>(base, oLj);
+    d.lj_tab = at<float4>(base, oUp + kUpLj);
     d.dbg_n = at<long long>(base, oDbg);
 
-    // per-call inputs of the scratch; zero what the kernels expect zeroed
+    // per-call inputs of the scratch in one copy, what the kernels expect
+    // zeroed in one memset, and the kernels of nb_step: 7 operations on the
+    // stream less than a copy or memset per array and nb_build_cells +
+    // nb_forces (with the fits kept, fit_ewald, a call for 900 atoms took
+    // 265 us and takes 88 us)
     cudaStream_t s = c.stream;
-    cudaError_t e = cudaMemcpyAsync(d.sys, &h_sys, sizeof(SysDesc), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.atom_sys, 0, sizeof(int) * N, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.col_sys, 0, sizeof(int) * C, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d.part_orig, h_part, sizeof(int) * N * K, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d.lj_tab, h_lj, sizeof(float4) * T * T, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.status, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.col_count, 0, sizeof(int) * (C + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.tslot, 0, sizeof(int) * c.slot_cap, s);
-    if (e == cudaSuccess) e = launch_build(&c, d_pos);
-    if (e == cudaSuccess) e = launch_forces(&c, d_pos, d_q, d_type, d_F, d_energy, d_virial, false);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaError_t e = cudaMemcpyAsync(base + oUp, h_up, up_part + sizeof(int) * N * K, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.status, 0, 16 + sizeof(int) * (2 * C + 1), s);
+    // as nb_step: charges and types packed by the column sort
+    if (e == cudaSuccess) e = launch_build_cells(&c, d_pos, d_q, d_type);
+    if (e == cudaSuccess) e = launch_build_lists(&c);
+    if (e == cudaSuccess) e = launch_forces_packed(&c, d_F, d_energy, d_virial, false, false, false);
     int h = 0;
-    if (e == cudaSuccess) e = cudaMemcpy(&h, d.status, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d.status, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     c.d = DevBuffers();  // the scratch belongs to the static array, not to c
     if (e != cudaSuccess) return NB_ERR_CUDA;
     if (h & ST_NONFINITE) return NB_ERR_NONFINITE;
