@@ -309,7 +309,7 @@ nb_status nb_step(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32
     // sorted atoms) is forked before the lists, beside the list and force kernels
     cudaError_t e = launch_build_cells(ctx, d_pos, d_q, d_type);
     const bool pme = ctx->pme != nullptr;
-    if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q);
+    if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, true, true);
     if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
     if (e != cudaSuccess) return NB_ERR_CUDA;
     ctx->built = true;

@@ -203,6 +203,7 @@ struct ColPack {
     long long *sys_acc;  // [n_acc] per-system energy and virial sums
     int n_acc;
     int *work;           // the force kernels' work-unit counter
+    long long *pme_acc;  // [kPmeAcc] PME sums, zeroed too (null without PME)
     int *status;
 };
 
@@ -395,6 +396,7 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_colsort(
         if (c == 0) {
             for (int k = tid; k < pk.n_acc; k += blockDim.x) pk.sys_acc[k] = 0;
             if (tid == 0) *pk.work = 0;
+            if (pk.pme_acc && tid < kPmeAcc) pk.pme_acc[tid] = 0;
         }
     }
     __syncthreads();
@@ -1269,7 +1271,7 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
                        (const int *)d.atom_col, d.wpos, d.xyzq, d.tslot, d.perm, d.inv, d.bb, d.clus_sys, d.zbin,
                        ctx->group, d.col_grp, d.grp, d.clus_grp,
                        ColPack{d_q, d_type, ctx->pp.n_types, d.atom_t, d.facc, d.sys_acc, kTaskVals * ctx->n_sys,
-                               d.counts + 3, d.status});
+                               d.counts + 3, pme_sums(ctx), d.status});
     if (e != cudaSuccess) return e;
     ctx->built_group = ctx->group;
     return cudaGetLastError();

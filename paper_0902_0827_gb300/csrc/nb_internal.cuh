@@ -246,6 +246,21 @@ __device__ __forceinline__ float fixed_to_float(long long v)
     return v < 0 ? -f : f;
 }
 
+// The nearest fixed-point value (2^32) of an FP32, the bits of
+// __float2ll_rn(f * 2^32), without the 64-bit conversion: the multiple of 1/2
+// next to f by adding 1.5 2^22 (exact remainder, at most 1/4), the remainder
+// by a 32-bit conversion.  |f| < 2^20 here; anything else takes the conversion.
+__device__ __noinline__ inline long long float_to_fixed_wide(float f) { return __float2ll_rn(f * 4294967296.0f); }
+
+__device__ __forceinline__ long long float_to_fixed(float f)
+{
+    if (!(fabsf(f) < 1048576.0f)) return float_to_fixed_wide(f);
+    const float t = __fadd_rn(f, 6291456.0f);
+    const float r = __fsub_rn(f, __fsub_rn(t, 6291456.0f));
+    const int lo = __float2int_rn(__fmul_rn(r, 4294967296.0f));
+    return (long long)(__float_as_int(t) - 0x4AC00000) * 2147483648ll + lo;
+}
+
 // Programmatic dependent launch.  Every kernel of the library calls
 // pdl_entry() before it reads or writes anything that another kernel writes
 // (at its start, or after a prologue that only fills shared memory from
@@ -335,12 +350,11 @@ cudaError_t launch_adjoint_tile(nb_ctx *ctx, const double *d_dLdE, float *d_dpos
 // Smooth PME (nb_pme.cu): the reciprocal-space chain into the context's PME
 // force and energy sums; the sums' device arrays (NULL when PME is off).
 cudaError_t launch_pme(nb_ctx *ctx, const float *d_pos, const float *d_q);
-// the same chain forked onto the PME side stream, and the join back
-// sums: also the pair-correction energy and virial (the forces always)
-// side_first: launched on the side stream before the PME chain (work that
-// is independent of the short-range path, e.g. the MD step's bonded terms).
-cudaError_t launch_pme_fork(nb_ctx *ctx, const float *d_pos, const float *d_q, bool sums = true,
-                            cudaError_t (*side_first)(nb_ctx *, cudaStream_t, const float *) = nullptr);
+// the same chain forked onto the PME side stream, and the join back.
+// sums: also the pair-correction energy and virial (the forces always);
+// zeroed: the PME sums were zeroed by the column sort
+cudaError_t launch_pme_fork(nb_ctx *ctx, const float *d_pos, const float *d_q, bool sums = true, bool zeroed = false);
+long long *pme_sums(const nb_ctx *ctx);
 cudaError_t launch_pme_join(nb_ctx *ctx);
 void pme_free(nb_ctx *ctx);
 const long long *pme_forces_acc(const nb_ctx *ctx);

@@ -868,7 +868,7 @@ static cudaError_t md_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, 
         if (e == cudaSuccess) e = launch_bonded(ctx, M.bside, d_pos);
         if (e == cudaSuccess) e = cudaEventRecord(M.bjoin, M.bside);
     }
-    if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, sums);
+    if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, sums, true);
     if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
     if (e != cudaSuccess) return e;
     ctx->built = true;
