@@ -964,8 +964,8 @@ __device__ __forceinline__ void tile1_virial_unit(float (&wimg)[3], long long &w
 
 __host__ __device__ inline size_t tile1_warp_bytes() { return (size_t)kBatch1 * kCluster * (16 + 4); }
 
-template <int W, int RAD, bool VIRIAL, bool DEBUG>
-__global__ void __launch_bounds__(W * 32, ACENB_TILE_MIN_BLOCKS * kTileWarps / W) k_force1(ForceArgs A, int parts,
+template <int W, int MB, int RAD, bool VIRIAL, bool DEBUG>
+__global__ void __launch_bounds__(W * 32, MB) k_force1(ForceArgs A, int parts,
                                                                                         int n_first)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1815,47 +1815,64 @@ static void launch_force_g(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
                blocks * kTileWarps);
 }
 
-// Blocks of W warps of k_force1 that an SM holds (-1: not asked yet; the
+// Blocks of an instance of k_force1 that an SM holds (-1: not asked yet; the
 // answer depends on the context's type count only and is kept there).
-template <int W, int RAD, bool VIRIAL, bool DEBUG>
-static int force1_resident(nb_ctx *ctx, size_t smem)
+template <int W, int MB, int RAD, bool VIRIAL, bool DEBUG>
+static int force1_resident(nb_ctx *ctx)
 {
-    int &r = ctx->force1_res[W == 4 ? 0 : 1][RAD][(VIRIAL ? 1 : 0) + (DEBUG ? 2 : 0)];
+    int &r = ctx->force1_res[W == 8 ? 0 : (MB == 8 ? 2 : 1)][RAD][(VIRIAL ? 1 : 0) + (DEBUG ? 2 : 0)];
     if (r >= 0) return r;
     static std::atomic<unsigned long long> optin{0};
-    smem_optin_once(k_force1<W, RAD, VIRIAL, DEBUG>, ctx->device, 200 * 1024, optin);
+    smem_optin_once(k_force1<W, MB, RAD, VIRIAL, DEBUG>, ctx->device, 200 * 1024, optin);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_force1<W, RAD, VIRIAL, DEBUG>, W * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_force1<W, MB, RAD, VIRIAL, DEBUG>, W * 32,
+                                                  lj_table_bytes(ctx->pp.n_types) + W * tile1_warp_bytes());
     return r = n;
 }
 
-template <int W, int RAD, bool VIRIAL, bool DEBUG>
-static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, int resident, size_t smem, bool beside_pme)
+template <int W, int MB, int RAD, bool VIRIAL, bool DEBUG>
+static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     constexpr int per = kTileWarps / W;  // blocks of W warps in the tuning's unit of kTileWarps warps
+    const int resident = force1_resident<W, MB, RAD, VIRIAL, DEBUG>(ctx);
+    // the tuning's default of 3 (24 warps) means all that fit of the smaller budget
+    const int want = W * MB > 24 && ctx->tune.blocks_per_sm >= 3 ? MB : ctx->tune.blocks_per_sm * per;
     // beside PME 8 of the 24 warps' room is left: 109.4 us a step at 23,500
     // atoms (4: 110.2, 12: 116, none: 121)
-    const int per_sm = std::max(1, std::min(ctx->tune.blocks_per_sm * per, resident) - (beside_pme ? per : 0));
+    const int per_sm = std::max(1, std::min(want, resident) - (beside_pme ? per : 0));
     const int parts = ctx->tune.list_split > 0 ? ctx->tune.list_split : kDefaultListSplit;
     const int blocks = ctx->num_sms * per_sm;
-    launch_pdl(k_force1<W, RAD, VIRIAL, DEBUG>, dim3(blocks), dim3(W * 32), smem, ctx->stream, A, parts, blocks * W);
+    launch_pdl(k_force1<W, MB, RAD, VIRIAL, DEBUG>, dim3(blocks), dim3(W * 32),
+               lj_table_bytes(A.P.n_types) + W * tile1_warp_bytes(), ctx->stream, A, parts, blocks * W);
 }
 
-// Blocks of 4 warps: they start and end in smaller steps than blocks of 8
-// (the kernel before and the kernel after share the SM's registers with them
-// sooner): rebuild + forces 93.4 -> 90.6 us at 23,500 atoms, 53.2 -> 51.2 us
-// at 6,144, the same at 999,999.  Each block holds the type-pair table, so
-// with many types (above about 26) an SM holds fewer warps in blocks of 4
-// than in blocks of 8, and blocks of 8 are taken.
+// Which instance.  Blocks of 4 warps start and end in smaller steps than
+// blocks of 8 (the kernel before and the kernel after share the SM's registers
+// with them sooner): rebuild + forces 93.4 -> 90.6 us at 23,500 atoms,
+// 53.2 -> 51.2 us at 6,144.  Each block holds the type-pair table, so with many
+// types (above about 26) an SM holds fewer warps in blocks of 4 than in blocks
+// of 8, and blocks of 8 are taken.  With 64 registers (a few spills) an SM
+// holds 32 warps instead of 24, which pays once every warp has kMinRounds
+// units (the longer units of fuller SMs make the end of a launch longer):
+// 1979 -> 1933 us at 999,999 atoms, 915 -> 904 us for 64 boxes, 110.6 -> 109.3
+// at 39,000, but 90.6 -> 93.1 us at 23,500.  The tabulated form waits for its
+// loads and always takes the fuller SMs (28 warps instead of 24: 95.9 -> 90.9 us
+// at 20,001 atoms).
+constexpr int kMinRounds = 4;
+
 template <int RAD, bool VIRIAL, bool DEBUG>
 static void launch_force_1(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
-    const size_t table = lj_table_bytes(A.P.n_types);
-    const size_t smem4 = table + 4 * tile1_warp_bytes(), smem8 = table + 8 * tile1_warp_bytes();
-    const int r4 = force1_resident<4, RAD, VIRIAL, DEBUG>(ctx, smem4);
-    const int r8 = force1_resident<8, RAD, VIRIAL, DEBUG>(ctx, smem8);
-    if (r4 >= 2 * r8) launch_force_1w<4, RAD, VIRIAL, DEBUG>(ctx, A, r4, smem4, beside_pme);
-    else launch_force_1w<8, RAD, VIRIAL, DEBUG>(ctx, A, r8, smem8, beside_pme);
+    if constexpr (!DEBUG) {
+        const int64_t units = kListSegs * ctx->clus_cap;
+        const bool rounds = !beside_pme && units >= (int64_t)kMinRounds * 32 * ctx->num_sms;
+        if ((RAD == 2 || rounds) && force1_resident<4, 8, RAD, VIRIAL, DEBUG>(ctx) >= 8)
+            return launch_force_1w<4, 8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+        if constexpr (RAD != 2)
+            if (force1_resident<4, 6, RAD, VIRIAL, DEBUG>(ctx) >= 2 * force1_resident<8, 3, RAD, VIRIAL, DEBUG>(ctx))
+                return launch_force_1w<4, 6, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+    }
+    launch_force_1w<8, 3, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
 }
 
 template <int RAD, bool VIRIAL, bool DEBUG>
@@ -1921,7 +1938,6 @@ static ForceArgs make_args(nb_ctx *ctx)
     A.dbg_ij = d.dbg_ij;
     A.dbg_cap = d.dbg_cap;
     A.P = ctx->pp;
-    A.C = make_const2(ctx->pp);
     return A;
 }
 
@@ -1963,6 +1979,7 @@ cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, doub
 {
     auto &d = ctx->d;
     ForceArgs A = make_args(ctx);
+    A.C = make_const2(ctx->pp);
     A.facc = d.facc;
     const bool ewald = ctx->pp.ewald != 0;
     const bool virial = d_virial != nullptr;

@@ -197,8 +197,9 @@ struct nb_ctx {
     int device = 0;
     int num_sms = 0;
     // resident blocks per SM of the single-cluster force kernel's instances
-    // (block size, radial functions, virial / debug), -1: not asked yet
-    int force1_res[2][3][4] = {{{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}},
+    // (block shape, radial functions, virial / debug), -1: not asked yet
+    int force1_res[3][3][4] = {{{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}},
+                               {{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}},
                                {{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}}};
     bool built = false;
     bool host_inputs = false;      // the step's charges and types were in host memory at the last query
