@@ -49,18 +49,16 @@ __global__ void k_tab_finalize(int T, const long long *__restrict__ acc, double 
     if (deps) deps[k] = (double)e * sc;
 }
 
-// Lorentz-Berthelot chain from type-pair to per-type gradients: one warp per
-// type, its lanes over the partners (a fixed order of the sums).  One thread
-// per type took 47 us for 22 types: a square root and a division in FP64 per
-// partner, one after the other; side by side they take 4.
-__global__ void __launch_bounds__(32) k_type_grad(int T, const float *__restrict__ eps, const double *__restrict__ gsig_tab,
-                                                  const double *__restrict__ geps_tab, double *__restrict__ gsig,
-                                                  double *__restrict__ geps)
+// Lorentz-Berthelot chain from type-pair to per-type gradients (one thread
+// per type; T <= 64).
+__global__ void k_type_grad(int T, const float *__restrict__ eps, const double *__restrict__ gsig_tab,
+                            const double *__restrict__ geps_tab, double *__restrict__ gsig, double *__restrict__ geps)
 {
     pdl_entry();
-    const int t = blockIdx.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= T) return;
     double gs = 0.0, ge = 0.0;
-    for (int b = threadIdx.x; b < T; b += 32) {
+    for (int b = 0; b < T; ++b) {
         const int k = t * T + b;
         if (b == t) {
             gs += gsig_tab[k];
@@ -70,21 +68,14 @@ __global__ void __launch_bounds__(32) k_type_grad(int T, const float *__restrict
             if (eps[b] != 0.0f) ge += geps_tab[k] * (double)eps[b] / (2.0 * sqrt((double)eps[t] * (double)eps[b]));
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        gs += __shfl_xor_sync(0xffffffffu, gs, o);
-        ge += __shfl_xor_sync(0xffffffffu, ge, o);
-    }
-    if (threadIdx.x == 0) {
-        gsig[t] = gs;
-        geps[t] = eps[t] == 0.0f ? __longlong_as_double(0x7ff8000000000000ll) : ge;
-    }
+    gsig[t] = gs;
+    geps[t] = eps[t] == 0.0f ? __longlong_as_double(0x7ff8000000000000ll) : ge;
 }
 
 cudaError_t launch_type_grad(nb_ctx *ctx, const double *gsig_tab, const double *geps_tab, double *gsig, double *geps)
 {
     const int T = ctx->pp.n_types;
-    launch_pdl(k_type_grad, dim3(T), dim3(32), 0, ctx->stream, T, ctx->d.eps_type, gsig_tab, geps_tab, gsig, geps);
+    launch_pdl(k_type_grad, dim3(1), dim3(64), 0, ctx->stream, T, ctx->d.eps_type, gsig_tab, geps_tab, gsig, geps);
     return cudaGetLastError();
 }
 
