@@ -1854,23 +1854,25 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 // of 8, and blocks of 8 are taken.  With 64 registers (a few spills) an SM
 // holds 32 warps instead of 24, which pays once every warp has kMinRounds
 // units (the longer units of fuller SMs make the end of a launch longer):
-// 1979 -> 1933 us at 999,999 atoms, 915 -> 904 us for 64 boxes, 110.6 -> 109.3
-// at 39,000, but 90.6 -> 93.1 us at 23,500.  The tabulated form waits for its
-// loads and always takes the fuller SMs (28 warps instead of 24: 95.9 -> 90.9 us
-// at 20,001 atoms).
+// 1976 -> 1928 us at 999,999 atoms, 511 -> 503 at 240,000, 914 -> 903 for 64
+// boxes, 110.7 -> 109.2 at 39,003, but 90.6 -> 93.1 us at 23,500.  The
+// tabulated form does not take it: 80.9 -> 83.3 us at 20,001 atoms, 129.0 ->
+// 131.9 at 39,003, 262 -> 268 at 90,000 (its loads go to L1 and L2, which more
+// warps share).
 constexpr int kMinRounds = 4;
 
 template <int RAD, bool VIRIAL, bool DEBUG>
 static void launch_force_1(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     if constexpr (!DEBUG) {
-        const int64_t units = kListSegs * ctx->clus_cap;
-        const bool rounds = !beside_pme && units >= (int64_t)kMinRounds * 32 * ctx->num_sms;
-        if ((RAD == 2 || rounds) && force1_resident<4, 8, RAD, VIRIAL, DEBUG>(ctx) >= 8)
-            return launch_force_1w<4, 8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
-        if constexpr (RAD != 2)
-            if (force1_resident<4, 6, RAD, VIRIAL, DEBUG>(ctx) >= 2 * force1_resident<8, 3, RAD, VIRIAL, DEBUG>(ctx))
-                return launch_force_1w<4, 6, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+        if constexpr (RAD != 2) {
+            const int64_t units = kListSegs * ctx->clus_cap;
+            const bool rounds = !beside_pme && units >= (int64_t)kMinRounds * 32 * ctx->num_sms;
+            if (rounds && force1_resident<4, 8, RAD, VIRIAL, DEBUG>(ctx) >= 8)
+                return launch_force_1w<4, 8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+        }
+        if (force1_resident<4, 6, RAD, VIRIAL, DEBUG>(ctx) >= 2 * force1_resident<8, 3, RAD, VIRIAL, DEBUG>(ctx))
+            return launch_force_1w<4, 6, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
     }
     launch_force_1w<8, 3, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
 }
