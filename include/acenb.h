@@ -101,7 +101,8 @@ typedef struct {
 
 /* Tuning knobs (chosen by the autotuner; defaults are safe). */
 typedef struct {
-    int32_t blocks_per_sm;  /* blocks per SM of the forward kernel's persistent grid, 1..8 */
+    int32_t blocks_per_sm;  /* persistent grid of the forward kernel, in units of 8 warps per SM, 1..8 (at most what
+                               fits; from 3 on, all that fits where the kernel runs with 64 registers) */
     int32_t stage_capacity; /* no effect (both kernels stage their lists in 32-entry batches);
                                validated as 16..512, multiple of 4 */
     int32_t list_capacity;  /* entries of an i-group's list (its share of the cluster pairs:
@@ -248,10 +249,11 @@ nb_status nb_debug_pairs(nb_ctx *ctx, int32_t *h_ij, int64_t cap, int64_t *n, in
 
 /* nb_debug_fill - tile fill of the last nb_debug_pairs run: *tiles receives
  * the number of 8 x 8 cluster-pair tiles the forward kernel visited and
- * *halves the number of 4 x 8 tile halves whose pair arithmetic ran (at
- * least one of their 32 pairs inside the cutoff and not excluded).  With the
- * pair count n of nb_debug_pairs, n / (64 tiles) is the tile fill and
- * n / (32 halves) the fraction of evaluated lanes doing useful work.
+ * *halves the number of 4 x 8 tile halves with at least one of their 32
+ * pairs inside the cutoff and not excluded.  With the pair count n of
+ * nb_debug_pairs, n / (64 tiles) is the tile fill and n / (32 halves) the
+ * fill of those halves.  (The kernel for groups of one cluster evaluates both
+ * halves of a tile that has a pair, those for larger groups only these.)
  * Measurement export without a counterpart in the paper.  Synchronous. */
 nb_status nb_debug_fill(nb_ctx *ctx, int64_t *tiles, int64_t *halves);
 
