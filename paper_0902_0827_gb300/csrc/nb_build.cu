@@ -978,6 +978,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
     if (!BESIDE) pdl_trigger();
     zero_histogram(A);
     if (g >= A.counts[4]) return;  // the whole warp
+    __syncwarp();  // every word of the map is cleared before any lane sets a bit
     const unsigned lt = (1u << lane) - 1u;
     int *s_col = s_col_all[w];
     int4 *s_ci = s_ci_all[w];
