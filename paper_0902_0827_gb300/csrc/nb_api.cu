@@ -311,7 +311,10 @@ nb_status nb_step(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32
     const bool pme = ctx->pme != nullptr;
     if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, true, true);
     if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
-    if (e != cudaSuccess) return NB_ERR_CUDA;
+    if (e != cudaSuccess) {
+        abandon_build(ctx, e);
+        return NB_ERR_CUDA;
+    }
     ctx->built = true;
     e = launch_forces_packed(ctx, d_F, d_energy, d_virial, false, pme, pme);
     return e == cudaSuccess ? NB_OK : NB_ERR_CUDA;

@@ -1247,6 +1247,36 @@ bool bins_elsewhere(nb_ctx *ctx, const float *d_q)
     return ctx->n_sys == 1 && ctx->n_cols <= kDirectCols && !inputs_in_host_memory(ctx, d_q);
 }
 
+// A second set of counts on top of the first would overflow the sorted arrays
+// (every atom staged twice), so the counts of a build whose lists were not
+// launched are cleared at once, in stream order: a graph captured earlier finds
+// them zero too.  The error is taken off the runtime (a later call would
+// report it again), and the lists no longer belong to the sorted atoms, unless
+// the stream is being captured and nothing has run.  Under a capture that the
+// error has ended the clearing is refused; then, as with any other refusal, the
+// next build clears.  What PME kernels were launched read the sorted atoms: the
+// stream waits for them.
+cudaError_t abandon_build(nb_ctx *ctx, cudaError_t e)
+{
+    cudaGetLastError();
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs == cudaStreamCaptureStatusNone) ctx->built = false;
+    if (ctx->pme) pme_rejoin(ctx);
+    ctx->hist_dirty = cudaMemsetAsync(ctx->d.col_count, 0, sizeof(int) * (2 * (size_t)ctx->n_cols + 1), ctx->stream) !=
+                      cudaSuccess;
+    cudaGetLastError();
+    return e;
+}
+
+cudaError_t ready_histogram(nb_ctx *ctx)
+{
+    if (!ctx->hist_dirty) return cudaSuccess;
+    const cudaError_t e =
+        cudaMemsetAsync(ctx->d.col_count, 0, sizeof(int) * (2 * (size_t)ctx->n_cols + 1), ctx->stream);
+    ctx->hist_dirty = e != cudaSuccess;
+    return e;
+}
+
 cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type, bool binned)
 {
     auto &d = ctx->d;
@@ -1255,11 +1285,11 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
     const bool host_in = !binned && d_q && d.atom_t && inputs_in_host_memory(ctx, d_q);
     // the column counts are zero here: zeroed at create and by the previous
     // build (its list kernel, or the scan of its binning kernel, which leaves
-    // a copy for the sort)
+    // a copy for the sort; abandon_build when it got to neither)
     const int direct = ctx->n_cols <= kDirectCols ? 1 : 0;
     const int tb = 256;
-    cudaError_t e = cudaSuccess;
-    if (!binned)
+    cudaError_t e = binned ? cudaSuccess : ready_histogram(ctx);
+    if (!binned && e == cudaSuccess)
         e = launch_pdl_split(ctx->pme, k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, bin_args(ctx),
                              (const int *)d.atom_sys, ctx->n_cols, ctx->n_sys, d.col_slot, d.counts, ctx->group, d.col_grp,
                              1 - direct,
@@ -1318,8 +1348,9 @@ cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme)
 
 cudaError_t launch_build(nb_ctx *ctx, const float *d_pos)
 {
-    const cudaError_t e = launch_build_cells(ctx, d_pos);
-    return e != cudaSuccess ? e : launch_build_lists(ctx);
+    cudaError_t e = launch_build_cells(ctx, d_pos);
+    if (e == cudaSuccess) e = launch_build_lists(ctx);
+    return e == cudaSuccess ? e : abandon_build(ctx, e);
 }
 
 }  // namespace acenb

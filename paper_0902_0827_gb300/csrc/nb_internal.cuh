@@ -203,6 +203,7 @@ struct nb_ctx {
                                {{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}}};
     bool built = false;
     bool host_inputs = false;      // the step's charges and types were in host memory at the last query
+    bool hist_dirty = false;       // an abandoned build's column counts could not be cleared yet
     acenb::PairParams pp{};
     nb_tuning tune{};
     std::vector<acenb::SysDesc> sys_h;
@@ -333,6 +334,11 @@ cudaError_t launch_build(nb_ctx *ctx, const float *d_pos);
 // bins_elsewhere: one system, no scan, charges in device memory)
 cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q = nullptr,
                                const int32_t *d_type = nullptr, bool binned = false);
+// a build that failed on the host behind its binning: clears the counts that its
+// list kernel would have cleared; returns e
+cudaError_t abandon_build(nb_ctx *ctx, cudaError_t e);
+// before anything bins: the column counts are zero
+cudaError_t ready_histogram(nb_ctx *ctx);
 BinArgs bin_args(const nb_ctx *ctx);
 bool bins_elsewhere(nb_ctx *ctx, const float *d_q);
 // beside_pme: the PME chain was forked before and is to run beside the lists
@@ -357,6 +363,8 @@ cudaError_t launch_pme(nb_ctx *ctx, const float *d_pos, const float *d_q);
 cudaError_t launch_pme_fork(nb_ctx *ctx, const float *d_pos, const float *d_q, bool sums = true, bool zeroed = false);
 long long *pme_sums(const nb_ctx *ctx);
 cudaError_t launch_pme_join(nb_ctx *ctx);
+// the context's stream waits for whatever was launched on the PME streams (after an error)
+void pme_rejoin(nb_ctx *ctx);
 void pme_free(nb_ctx *ctx);
 const long long *pme_forces_acc(const nb_ctx *ctx);
 const long long *pme_sums_acc(const nb_ctx *ctx);

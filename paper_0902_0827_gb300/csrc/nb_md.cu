@@ -870,7 +870,7 @@ static cudaError_t md_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, 
     }
     if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, sums, true);
     if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return abandon_build(ctx, e);
     ctx->built = true;
     e = launch_forces_packed(ctx, unpack ? M.Fnb : nullptr, unpack ? M.enb : nullptr, nullptr, false, pme, pme);
     if (e != cudaSuccess) return e;
@@ -1052,6 +1052,7 @@ extern "C" nb_status nb_md_step(nb_ctx *ctx, float *d_pos, float *d_vel, const f
     // the half-steps bin the atoms they move, where the binning needs no scan
     const bool binned = bins_elsewhere(ctx, d_q);
     const BinArgs bin = binned ? bin_args(ctx) : BinArgs{};
+    if (binned) e = ready_histogram(ctx);
     for (int s = 0; s < n_steps && e == cudaSuccess; ++s) {
         if (s == 0)
             e = launch_pdl_split(ctx->pme, k_md_first, dim3(ib), dim3(64), 0, st, A, bin);

@@ -864,6 +864,13 @@ cudaError_t launch_pme_fork(nb_ctx *ctx, const float *d_pos, const float *d_q, b
 
 long long *pme_sums(const nb_ctx *ctx) { return ctx->pme ? ctx->pme->acc : nullptr; }
 
+void pme_rejoin(nb_ctx *ctx)
+{
+    PmeState &P = *ctx->pme;
+    if (cudaEventRecord(P.join, P.side) == cudaSuccess) cudaStreamWaitEvent(ctx->stream, P.join, 0);
+    if (cudaEventRecord(P.corr, P.cside) == cudaSuccess) cudaStreamWaitEvent(ctx->stream, P.corr, 0);
+}
+
 cudaError_t launch_pme_join(nb_ctx *ctx)
 {
     return cudaStreamWaitEvent(ctx->stream, ctx->pme->join, 0);
