@@ -149,6 +149,13 @@ nb_status nb_create_batch(int32_t n_sys, const nb_params *params, void *cuda_str
     int64_t N = 0;
     for (int s = 0; s < n_sys; ++s) N += params[s].n_atoms;
     if (N > (int64_t)1 << 28) return NB_ERR_UNSUPPORTED;
+    int64_t columns = 0;
+    for (int s = 0; s < n_sys; ++s) {
+        SysDesc S;
+        init_sysdesc(params[s], S, 0, 0, 0);
+        columns += (int64_t)S.nx * S.ny;
+    }
+    if ((N + (kCluster - 1) * columns) / kCluster + 1 > kMaxClusterCap) return NB_ERR_UNSUPPORTED;
 
     nb_ctx *c = new (std::nothrow) nb_ctx();
     if (!c) return NB_ERR_OOM;

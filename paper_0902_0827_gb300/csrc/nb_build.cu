@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
                                     rec[q2] = r;
                                 }
                             }
-                            ent.y |= (uint32_t)slot << kMaskSlotBit;
+                            ent.y |= mask_field(A.group, slot, q < loc_cap ? q : -1, A.pool_base);
                         } else {
                             atomicOr(A.status, ST_CAPACITY);
                             ent.x &= ~kExclFlag;
@@ -987,7 +987,8 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
     const int K = A.K, np = kCluster * K;  // partner entries, at most 128
     const float inv_K = 1.0f / (float)K;
     // the partners of the group's atoms: three dependent loads, every round's
-    // in flight together (partner cluster << 7 | is14 << 6 | bit 8 a + jj)
+    // in flight together (partner cluster << 7 | is14 << 6 | bit 8 a + jj, all
+    // 32 bits: the cluster takes 25 of them; none: -1, no cluster's index)
     int pk[kPartnerBatch];
 #pragma unroll
     for (int r = 0; r < kPartnerBatch; ++r) {
@@ -1010,7 +1011,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
             int rr;
             const int a = div_small(r * 32 + lane, K, inv_K, rr);
             const int pc = v / kCluster;
-            pk[r] = (pc << 7) | ((pk[r] & 1) << 6) | (a * kCluster + (v & (kCluster - 1)));
+            pk[r] = (int)((unsigned)pc << 7) | ((pk[r] & 1) << 6) | (a * kCluster + (v & (kCluster - 1)));
             atomicOr(&s_map[(pc >> 5) & (kMapWords - 1)], 1u << (pc & 31));
         }
     }
@@ -1149,7 +1150,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
                     for (int r = 0; r < kPartnerBatch; ++r) {
                         if (r * 32 >= np) break;  // the whole warp
                         const int v = pk[r];
-                        if (v >= 0 && (v >> 7) == JL) {
+                        if (v != -1 && (int)((unsigned)v >> 7) == JL) {
                             const int bit = v & 63;
                             const unsigned m = 1u << (bit & 31);
                             if (v & 64) {
@@ -1190,7 +1191,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(G
                         if (slot < A.mask_cap) {
                             A.gmask[slot] = make_ulonglong2(ex, s14);
                             ent.x |= kExclFlag;
-                            ent.y |= (uint32_t)slot << kMaskSlotBit;
+                            ent.y |= (uint32_t)slot << mask_bit(1);
                         } else {
                             atomicOr(A.status, ST_CAPACITY);
                         }
@@ -1330,6 +1331,8 @@ cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme)
     A.status = d.status;
     A.pool_base = mask_pool_base(ctx->clus_cap);
     A.mask_cap = ctx->mask_cap;
+    if (ctx->built_group == 8)  // what 24 bits name of the pool
+        A.mask_cap = std::min<long long>(A.mask_cap, A.pool_base + (1 << 24) - kOwnRecs8);
     A.K = ctx->K;
     A.rcm = ctx->pp.rc + ctx->pp.list_margin;
     A.cap = ctx->list_cap;

@@ -57,7 +57,18 @@ struct ForceArgs {
     const float4 *lj_d;      // [T*T] 48 eps sig^11, 24 eps sig^5, 4 sig^12, 4 sig^6
     long long *tab_acc;      // [T*T*2] fixed-point dL/dsig_ab, dL/deps_ab (each unique pair in one order)
     long long *gacc;         // [S*4] fixed-point dL/dx, dL/dq in sorted order (both atoms of each pair)
+    const ulonglong2 *pool8;  // groups of 8: where record number 0 of the pool's count would be
 };
+
+// The masks of a flagged entry of a group of G clusters, one pair per cluster
+// (own8: groups of 8, the group's first own record).
+template <int G>
+__device__ __forceinline__ const ulonglong2 *entry_record(const ForceArgs &A, uint32_t y, const ulonglong2 *own8)
+{
+    const uint32_t k = y >> mask_bit(G);
+    if constexpr (G == 8) return (k < kOwnRecs8 ? own8 : A.pool8) + k * 8ull;
+    return A.gmask + (unsigned long long)k * G;
+}
 
 __device__ __forceinline__ long long to_fixed(float v, int *status)
 {
@@ -460,8 +471,8 @@ __device__ __forceinline__ void tile_pair2(const ForceArgs &A, const float4 *__r
 template <int G, int RAD, bool VIRIAL, bool DEBUG, bool SPECIAL, bool IMG>
 __device__ __forceinline__ void tile_entry(const ForceArgs &A, const float4 *__restrict__ lj,
                                            const float4 *__restrict__ s_ix, const int *__restrict__ s_it,
-                                           const int *__restrict__ s_io, float4 *__restrict__ s_fi, uint2 ent,
-                                           float4 pjA, float4 pjB, int tjA, int tjB, int ia, int jb, int lane, float Lx,
+                                           const int *__restrict__ s_io, float4 *__restrict__ s_fi,
+                                           const ulonglong2 *own8, uint2 ent, float4 pjA, float4 pjB, int tjA, int tjB, int ia, int jb, int lane, float Lx,
                                            float Ly, float Lz, float &elj, float &ec, float (&wimg)[6], bool &ovf)
 {
     const int J = (int)(ent.x & kJMask);
@@ -473,9 +484,9 @@ __device__ __forceinline__ void tile_entry(const ForceArgs &A, const float4 *__r
     }
     const int jorigA = DEBUG ? __ldg(A.perm + (long long)J * kCluster + jb) : -1;
     const int jorigB = DEBUG ? __ldg(A.perm + (long long)J * kCluster + jb + 4) : -1;
-    const ulonglong2 *rec = SPECIAL ? A.gmask + (long long)(ent.y >> kMaskSlotBit) * G : nullptr;
+    const ulonglong2 *rec = SPECIAL ? entry_record<G>(A, ent.y, own8) : nullptr;
     float fjAx = 0.0f, fjAy = 0.0f, fjAz = 0.0f, fjBx = 0.0f, fjBy = 0.0f, fjBz = 0.0f;
-    for (unsigned cm = ent.y & 0xFFu; cm; cm &= cm - 1u) {
+    for (unsigned cm = ent.y & ((1u << mask_bit(G)) - 1u); cm; cm &= cm - 1u) {
         const int c = __ffs(cm) - 1;
         const int ii = c * kCluster + ia;
         const ulonglong2 gm = SPECIAL ? rec[c] : make_ulonglong2(0ull, 0ull);
@@ -603,6 +614,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
         if (U.e_begin < U.e_end) {
             const int2 gr = __ldg(A.grp + U.g);
             const int c0 = gr.x, ncl = gr.y;
+            const ulonglong2 *own8 = G == 8 ? A.gmask + (long long)c0 * kMaskRecsPerCluster * 8 : nullptr;
             const int sys_id = __ldg(A.clus_sys + c0);
             if (sys_id != cur_sys) {
                 if (!DEBUG && cur_sys >= 0) {
@@ -667,7 +679,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                     plain &= plain - 1u;
                     const uint2 ent = make_uint2(__shfl_sync(kFull, my.x, k), __shfl_sync(kFull, my.y, k));
                     tile_entry<G, RAD, VIRIAL, DEBUG, false, false>(
-                        A, lj, s_ix, s_it, s_io, s_fi, ent, sjp[swz(k, jb)], sjp[swz(k, jb + 4)], sjt[swz(k, jb)],
+                        A, lj, s_ix, s_it, s_io, s_fi, own8, ent, sjp[swz(k, jb)], sjp[swz(k, jb + 4)], sjt[swz(k, jb)],
                         sjt[swz(k, jb + 4)], ia, jb, lane, Lx, Ly, Lz, elj, ec, wimg, ovf);
                 }
                 while (other) {
@@ -680,16 +692,16 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
                     const bool special = (ent.x & kExclFlag) != 0u;
                     if (img) {
                         if (special)
-                            tile_entry<G, RAD, VIRIAL, DEBUG, true, true>(A, lj, s_ix, s_it, s_io, s_fi, ent, pjA, pjB,
-                                                                         tjA, tjB, ia, jb, lane, Lx, Ly, Lz, elj, ec,
+                            tile_entry<G, RAD, VIRIAL, DEBUG, true, true>(A, lj, s_ix, s_it, s_io, s_fi, own8, ent, pjA,
+                                                                         pjB, tjA, tjB, ia, jb, lane, Lx, Ly, Lz, elj, ec,
                                                                          wimg, ovf);
                         else
-                            tile_entry<G, RAD, VIRIAL, DEBUG, false, true>(A, lj, s_ix, s_it, s_io, s_fi, ent, pjA,
-                                                                          pjB, tjA, tjB, ia, jb, lane, Lx, Ly, Lz, elj,
+                            tile_entry<G, RAD, VIRIAL, DEBUG, false, true>(A, lj, s_ix, s_it, s_io, s_fi, own8, ent,
+                                                                          pjA, pjB, tjA, tjB, ia, jb, lane, Lx, Ly, Lz, elj,
                                                                           ec, wimg, ovf);
                     } else {
-                        tile_entry<G, RAD, VIRIAL, DEBUG, true, false>(A, lj, s_ix, s_it, s_io, s_fi, ent, pjA, pjB,
-                                                                      tjA, tjB, ia, jb, lane, Lx, Ly, Lz, elj, ec, wimg,
+                        tile_entry<G, RAD, VIRIAL, DEBUG, true, false>(A, lj, s_ix, s_it, s_io, s_fi, own8, ent, pjA,
+                                                                      pjB, tjA, tjB, ia, jb, lane, Lx, Ly, Lz, elj, ec, wimg,
                                                                       ovf);
                     }
                 }
@@ -892,7 +904,7 @@ __device__ __forceinline__ void tile1_entry(const ForceArgs &A, const float4 *__
     bool inA = r2A < A.P.rc2, inB = r2B < A.P.rc2;
     bool s14A = false, s14B = false;
     if (SPECIAL) {  // exclusion bitmask of the tile: bit 8 i + j
-        const ulonglong2 m = A.gmask[ent.y >> kMaskSlotBit];  // records of one cluster
+        const ulonglong2 m = A.gmask[ent.y >> mask_bit(1)];  // records of one cluster
         const int bA = ih * kCluster + jj, bB = bA + 4 * kCluster;
         inA = inA && !((m.x >> bA) & 1ull);
         inB = inB && !((m.x >> bB) & 1ull);
@@ -1143,8 +1155,8 @@ __host__ __device__ inline size_t adj_warp_bytes(int G)
 template <int G, int RAD>
 __device__ __forceinline__ void adj_entry(const ForceArgs &A, const AdjTables &tab, const float4 *__restrict__ s_ix,
                                           const int *__restrict__ s_it, const float4 *__restrict__ s_ig,
-                                          float4 *__restrict__ s_ai, uint2 ent, float4 pjA, float4 pjB, float4 gjA,
-                                          float4 gjB, int tjA, int tjB, float gE_lj, float gE_c, int ia, int jb,
+                                          float4 *__restrict__ s_ai, const ulonglong2 *own8, uint2 ent, float4 pjA,
+                                          float4 pjB, float4 gjA, float4 gjB, int tjA, int tjB, float gE_lj, float gE_c, int ia, int jb,
                                           int lane, float Lx, float Ly, float Lz, bool &ovf)
 {
     const int J = (int)(ent.x & kJMask);
@@ -1155,9 +1167,9 @@ __device__ __forceinline__ void adj_entry(const ForceArgs &A, const AdjTables &t
         if (((code >> 2) & 3u) == 1u) { pjA.y = __fsub_rn(pjA.y, Ly); pjB.y = __fsub_rn(pjB.y, Ly); }
         if ((code >> 4) == 1u) { pjA.z = __fsub_rn(pjA.z, Lz); pjB.z = __fsub_rn(pjB.z, Lz); }
     }
-    const ulonglong2 *rec = special ? A.gmask + (long long)(ent.y >> kMaskSlotBit) * G : nullptr;
+    const ulonglong2 *rec = special ? entry_record<G>(A, ent.y, own8) : nullptr;
     float jA[4] = {0.0f, 0.0f, 0.0f, 0.0f}, jB[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (unsigned cm = ent.y & 0xFFu; cm; cm &= cm - 1u) {
+    for (unsigned cm = ent.y & ((1u << mask_bit(G)) - 1u); cm; cm &= cm - 1u) {
         const int c = __ffs(cm) - 1;
         const int ii = c * kCluster + ia;
         float4 pi = s_ix[ii];
@@ -1260,6 +1272,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint(ForceArgs A, int par
         if (U.e_begin < U.e_end) {
             const int2 gr = __ldg(A.grp + U.g);
             const int c0 = gr.x, ncl = gr.y;
+            const ulonglong2 *own8 = G == 8 ? A.gmask + (long long)c0 * kMaskRecsPerCluster * 8 : nullptr;
             const int sys_id = __ldg(A.clus_sys + c0);
             if (sys_id != cur_sys) {
                 cur_sys = sys_id;
@@ -1305,7 +1318,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint(ForceArgs A, int par
                 __syncwarp();
                 for (int k = 0; k < ne; ++k) {
                     const uint2 ent = make_uint2(__shfl_sync(kFull, my.x, k), __shfl_sync(kFull, my.y, k));
-                    adj_entry<G, RAD>(A, tab, s_ix, s_it, s_ig, s_ai, ent, sjp[swz(k, jb)], sjp[swz(k, jb + 4)],
+                    adj_entry<G, RAD>(A, tab, s_ix, s_it, s_ig, s_ai, own8, ent, sjp[swz(k, jb)], sjp[swz(k, jb + 4)],
                                       sjg[swz(k, jb)], sjg[swz(k, jb + 4)], sjt[swz(k, jb)], sjt[swz(k, jb + 4)],
                                       gE_lj, gE_c, ia, jb, lane, Lx, Ly, Lz, ovf);
                 }
@@ -1403,7 +1416,7 @@ __device__ __forceinline__ void adj1_entry(const ForceArgs &A, const AdjTables &
     bool inA = r2A < A.P.rc2, inB = r2B < A.P.rc2;
     bool s14A = false, s14B = false;
     if (special) {  // exclusion bitmask of the tile: bit 8 i + j
-        const ulonglong2 m = A.gmask[ent.y >> kMaskSlotBit];
+        const ulonglong2 m = A.gmask[ent.y >> mask_bit(1)];
         const int bA = ih * kCluster + jj, bB = bA + 4 * kCluster;
         inA = inA && !((m.x >> bA) & 1ull);
         inB = inB && !((m.x >> bB) & 1ull);
@@ -1930,6 +1943,7 @@ static ForceArgs make_args(nb_ctx *ctx)
     A.glist = d.glist;
     A.glist_n = d.glist_n;
     A.gmask = d.gmask;
+    A.pool8 = d.gmask + (mask_pool_base(ctx->clus_cap) - kOwnRecs8) * 8;
     A.cap = ctx->list_cap;
     A.K = ctx->K;
     A.lj_tab = d.lj_tab;

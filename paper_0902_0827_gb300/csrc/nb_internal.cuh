@@ -38,12 +38,14 @@ __host__ __device__ inline bool is_real_coord(float x) { return x > -1.0e17f; }
 // Group list entry (uint2).  x: J (bits 0..24) | shift codes x,y,z (2 bits
 // each, bits 25..30: 0 none, 1 = j-side shift x_j - L, 2 = i-side shift
 // x_i - L) | mask flag (bit 31: the entry's tiles have exclusion masks).
-// y: the group's clusters in reach of J (bits 0..7, bit c = cluster c of the
-// group) | mask record (bits 8..31, when flagged).
+// y: the group's clusters in reach of J (low bits, one per cluster of the
+// group) | mask record (the bits above, when flagged; see mask_field).
 constexpr uint32_t kJMask = 0x01FFFFFFu;
 constexpr int kShiftBit = 25;
 constexpr uint32_t kExclFlag = 0x80000000u;
-constexpr int kMaskSlotBit = 8;
+// Clusters of a context, capacity: at most kJMask, so that every index fits
+// an entry and the list kernel's packed partners (index << 7, all ones: none).
+constexpr int64_t kMaxClusterCap = kJMask;
 
 // Device status bits (first error wins when reported).
 enum : int {
@@ -321,6 +323,19 @@ inline int64_t group_capacity(int64_t clus_cap) { return clus_cap + 1; }
 // them.
 inline int64_t mask_pool_base(int64_t clus_cap) { return clus_cap * kMaskRecsPerCluster; }
 inline int64_t mask_capacity(int64_t clus_cap) { return mask_pool_base(clus_cap) + clus_cap / 2 + 64; }
+// The mask record in an entry's y, above the group's cluster bits (1, 4 or 8).
+// The 31 or 28 bits of the smaller groups hold the record's index.  The 24 bits
+// of groups of 8 would name the records of 2.8 million clusters only: they
+// count the group's own records (own >= 0: the record's place among them) from
+// the group's first, then those of the pool.  (The same form for groups of 4
+// cost 0.5 % of a step.)
+constexpr int kOwnRecs8 = 8 * kMaskRecsPerCluster;
+__host__ __device__ constexpr int mask_bit(int group) { return group; }
+__host__ __device__ inline uint32_t mask_field(int group, long long slot, int own, long long pool_base)
+{
+    const long long k = group != 8 ? slot : (own >= 0 ? own : kOwnRecs8 + (slot - pool_base));
+    return (uint32_t)k << mask_bit(group);
+}
 // atoms per column staging row for a mean column population: twice the mean
 // and 32 more, in whole warps (rows that overflow are gathered by the column
 // sort's slow fallback)
