@@ -1851,8 +1851,11 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
     // the tuning's default of 3 (24 warps) means all that fit of the smaller budget
     const int want = W * MB > 24 && ctx->tune.blocks_per_sm >= 3 ? MB : ctx->tune.blocks_per_sm * per;
     // beside PME 8 of the 24 warps' room is left: 109.4 us a step at 23,500
-    // atoms (4: 110.2, 12: 116, none: 121)
-    const int per_sm = std::max(1, std::min(want, resident) - (beside_pme ? per : 0));
+    // atoms (4: 110.2, 12: 116, none: 121).  A smaller grid leaves it as it
+    // is: 8 and 16 warps asked for less another 8 took 199 and 134 us, as asked
+    // for 137 and 107
+    const int room = beside_pme ? std::max(resident - per, std::min(per, resident)) : resident;
+    const int per_sm = std::max(1, std::min(want, room));
     const int parts = ctx->tune.list_split > 0 ? ctx->tune.list_split : kDefaultListSplit;
     const int blocks = ctx->num_sms * per_sm;
     launch_pdl(k_force1<W, MB, RAD, VIRIAL, DEBUG>, dim3(blocks), dim3(W * 32),
