@@ -1848,8 +1848,8 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     constexpr int per = kTileWarps / W;  // blocks of W warps in the tuning's unit of kTileWarps warps
     const int resident = force1_resident<W, MB, RAD, VIRIAL, DEBUG>(ctx);
-    // the tuning's default of 3 (24 warps) means all that fit of the smaller budget
-    const int want = W * MB > 24 && ctx->tune.blocks_per_sm >= 3 ? MB : ctx->tune.blocks_per_sm * per;
+    // (the 64-register shape runs with blocks_per_sm 3, the default, or more: all that fit)
+    const int want = W * MB > 24 ? MB : ctx->tune.blocks_per_sm * per;
     // beside PME 8 of the 24 warps' room is left: 109.4 us a step at 23,500
     // atoms (4: 110.2, 12: 116, none: 121).  A smaller grid leaves it as it
     // is: 8 and 16 warps asked for less another 8 took 199 and 134 us, as asked
@@ -1867,8 +1867,13 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 // with them sooner): rebuild + forces 93.4 -> 90.6 us at 23,500 atoms,
 // 53.2 -> 51.2 us at 6,144.  Each block holds the type-pair table, so with many
 // types (above about 26) an SM holds fewer warps in blocks of 4 than in blocks
-// of 8, and blocks of 8 are taken.  With 64 registers (a few spills) an SM
-// holds 32 warps instead of 24, which pays once every warp has kMinRounds
+// of 8, and blocks of 8 are taken.  So are they for a grid of 8 warps per SM
+// (blocks_per_sm 1), whose blocks of 4 would not spread evenly over SMs that
+// hold six of them (164 us at 23,500 atoms, 139 with blocks of 8; beside PME
+// 137 and 141).  With 64 registers (a few spills) an SM
+// holds 32 warps instead of 24, which, where the grid is to fill the SM (a
+// smaller grid spreads unevenly here too: 2,875 us at 999,999 atoms with
+// blocks_per_sm 2, 2,307 with 80 registers), pays once every warp has kMinRounds
 // units (the longer units of fuller SMs make the end of a launch longer):
 // 1976 -> 1928 us at 999,999 atoms, 511 -> 503 at 240,000, 914 -> 903 for 64
 // boxes, 110.7 -> 109.2 at 39,003, but 90.6 -> 93.1 us at 23,500.  The
@@ -1883,11 +1888,13 @@ static void launch_force_1(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
     if constexpr (!DEBUG) {
         if constexpr (RAD != 2) {
             const int64_t units = kListSegs * ctx->clus_cap;
-            const bool rounds = !beside_pme && units >= (int64_t)kMinRounds * 32 * ctx->num_sms;
+            const bool rounds = !beside_pme && ctx->tune.blocks_per_sm >= 3 &&
+                                units >= (int64_t)kMinRounds * 32 * ctx->num_sms;
             if (rounds && force1_resident<4, 8, RAD, VIRIAL, DEBUG>(ctx) >= 8)
                 return launch_force_1w<4, 8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
         }
-        if (force1_resident<4, 6, RAD, VIRIAL, DEBUG>(ctx) >= 2 * force1_resident<8, 3, RAD, VIRIAL, DEBUG>(ctx))
+        const bool fours = beside_pme || ctx->tune.blocks_per_sm > 1;
+        if (fours && force1_resident<4, 6, RAD, VIRIAL, DEBUG>(ctx) >= 2 * force1_resident<8, 3, RAD, VIRIAL, DEBUG>(ctx))
             return launch_force_1w<4, 6, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
     }
     launch_force_1w<8, 3, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
