@@ -662,6 +662,11 @@ constexpr int kPartnerBatch = 4;  // rounds of partner loads in flight
 
 __host__ __device__ inline size_t glist_warp_ints(int K, int group) { return 2 * (size_t)kCluster * group * K; }
 
+// BESIDE: the PME chain, forked before this kernel, is to run beside it.  The
+// next kernel's blocks are then not let in early: the force kernel's would
+// take the registers that the PME spread needs, and hold them while they wait
+// for the lists.
+template <bool BESIDE>
 __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_glist(GListArgs A)
 {
     const unsigned FULL = 0xffffffffu;
@@ -673,7 +678,8 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
         s_hash_all[w][t] = -1;
         s_head_all[w][t] = kLinkEnd;
     }
-    pdl_entry();
+    pdl_wait();
+    if (!BESIDE) pdl_trigger();
     zero_histogram(A);
     if (g >= A.counts[4]) return;  // the whole warp
     const unsigned lt = (1u << lane) - 1u;
@@ -954,10 +960,7 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
 constexpr int kGList1MinBlocks = 8;
 constexpr int kMapWords = 32;  // partner-cluster map: 1,024 bits
 
-// BESIDE: the PME chain, forked before this kernel, is to run beside it.  The
-// next kernel's blocks are then not let in early: the force kernel's would
-// take the registers that the PME spread needs, and hold them while they wait
-// for the lists.  (With the equal shared-memory split of launch_pdl_split:
+// BESIDE: as for k_glist.  (With the equal shared-memory split of launch_pdl_split:
 // rebuild + forces with PME 125.5 -> 113.3 us at 23,500 atoms, the MD step
 // 127 -> 114 us; without the second force launch that used to follow the PME
 // chain, 109 and 106 us.)
@@ -1344,7 +1347,8 @@ cudaError_t launch_build_lists(nb_ctx *ctx, bool beside_pme)
     cudaError_t e = A.group == 1
                         ? launch_pdl_split(beside_pme, beside_pme ? k_glist1<true> : k_glist1<false>, dim3((unsigned)blocks),
                                      dim3(kGListWarps * 32), 0, ctx->stream, A)
-                        : launch_pdl(k_glist, dim3((unsigned)blocks), dim3(kGListWarps * 32), smem, ctx->stream, A);
+                        : launch_pdl_split(beside_pme, beside_pme ? k_glist<true> : k_glist<false>, dim3((unsigned)blocks),
+                                     dim3(kGListWarps * 32), smem, ctx->stream, A);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -1806,14 +1806,16 @@ static void smem_optin_once(Kernel kernel, int device, int bytes, std::atomic<un
 size_t tile_smem_bytes(int T, int G) { return lj_table_bytes(T) + (size_t)kTileWarps * tile_warp_bytes(G); }
 
 // beside_pme: the PME chain, forked before the list kernel, runs on its side
-// stream during this kernel; the persistent grid then leaves one block slot
-// (of kTileWarps warps) per SM free, so that the PME kernels run alongside
-// instead of after it.  Which block takes which unit does not change any
-// result.  (A second launch behind the PME chain that took units from the same
+// stream during the list kernel and this one.  The persistent grid for groups of
+// one cluster then leaves room for 8 warps per SM, so that the PME kernels run
+// alongside instead of after it; the kernels for larger groups, which hold
+// fewer warps anyway, take what the tuning asks for (23,500 atoms: 138 us a
+// step with groups of 4, 151 with a block less; 180 and 210 with groups of 8).
+// Which block takes which unit does not change any result.  (A second launch behind the PME chain that took units from the same
 // counter made up for a chain that started late; now that the chain starts
 // with the lists it costs 4 us of the PME step and 7 us of an MD step.)
 template <int G, int RAD, bool VIRIAL, bool DEBUG>
-static void launch_force_g(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
+static void launch_force_g(nb_ctx *ctx, const ForceArgs &A)
 {
     const size_t smem = tile_smem_bytes(A.P.n_types, G);
     static std::atomic<unsigned long long> optin{0};
@@ -1821,7 +1823,7 @@ static void launch_force_g(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
     // persistent grid: never more blocks than can be resident at once
     int resident = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_force<G, RAD, VIRIAL, DEBUG>, kTileWarps * 32, smem);
-    const int per_sm = std::max(1, std::min(ctx->tune.blocks_per_sm, resident) - (beside_pme ? 1 : 0));
+    const int per_sm = std::max(1, std::min(ctx->tune.blocks_per_sm, resident));
     const int parts = ctx->tune.list_split > 0 ? ctx->tune.list_split : kDefaultListSplit;
     const int blocks = ctx->num_sms * per_sm;
     launch_pdl(k_force<G, RAD, VIRIAL, DEBUG>, dim3(blocks), dim3(kTileWarps * 32), smem, ctx->stream, A, parts,
@@ -1904,8 +1906,8 @@ template <int RAD, bool VIRIAL, bool DEBUG>
 static void launch_force_t(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     if (ctx->built_group == 1) launch_force_1<RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
-    else if (ctx->built_group == 4) launch_force_g<4, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
-    else launch_force_g<8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
+    else if (ctx->built_group == 4) launch_force_g<4, RAD, VIRIAL, DEBUG>(ctx, A);
+    else launch_force_g<8, RAD, VIRIAL, DEBUG>(ctx, A);
 }
 
 // The packed constants of a parameter block.
