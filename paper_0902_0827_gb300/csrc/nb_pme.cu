@@ -815,10 +815,10 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     e = launch_pdl_split(true, k_pme_solve, dim3(sb), dim3(256), 0, st, half, g, pi2_over_a2, (const float *)P.gfac,
                          P.fq, P.acc);
     if (e != cudaSuccess) return e;
-    if (cufftSetStream(P.inv, st) != CUFFT_SUCCESS || cufftExecC2R(P.inv, (cufftComplex *)P.fq, P.grid) != CUFFT_SUCCESS)
-        return cudaErrorUnknown;
     e = cudaStreamWaitEvent(st, P.corr, 0);
     if (e != cudaSuccess) return e;
+    if (cufftSetStream(P.inv, st) != CUFFT_SUCCESS || cufftExecC2R(P.inv, (cufftComplex *)P.fq, P.grid) != CUFFT_SUCCESS)
+        return cudaErrorUnknown;
     constexpr int G = GatherLanes<N>::G;
     const int S = (int)ctx->slot_cap;
     const int gt = 256;
