@@ -317,13 +317,13 @@ nb_status nb_step(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32
     cudaError_t e = launch_build_cells(ctx, d_pos, d_q, d_type);
     const bool pme = ctx->pme != nullptr;
     if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, true, true);
-    if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
+    if (e == cudaSuccess) e = launch_build_lists(ctx, pme_beside(ctx));
     if (e != cudaSuccess) {
         abandon_build(ctx, e);
         return NB_ERR_CUDA;
     }
     ctx->built = true;
-    e = launch_forces_packed(ctx, d_F, d_energy, d_virial, false, pme, pme);
+    e = launch_forces_packed(ctx, d_F, d_energy, d_virial, false, pme, pme_beside(ctx));
     return e == cudaSuccess ? NB_OK : NB_ERR_CUDA;
 }
 

@@ -1294,13 +1294,13 @@ cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q
     const int tb = 256;
     cudaError_t e = binned ? cudaSuccess : ready_histogram(ctx);
     if (!binned && e == cudaSuccess)
-        e = launch_pdl_split(ctx->pme, k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, bin_args(ctx),
+        e = launch_pdl_split(pme_beside(ctx), k_bin, dim3((N + tb - 1) / tb), dim3(tb), 0, st, N, d_pos, bin_args(ctx),
                              (const int *)d.atom_sys, ctx->n_cols, ctx->n_sys, d.col_slot, d.counts, ctx->group, d.col_grp,
                              1 - direct,
                              host_in ? AtomPack{d_q, d_type, ctx->pp.n_types, d.atom_t}
                                      : AtomPack{nullptr, nullptr, 0, nullptr});
     if (e == cudaSuccess)
-        e = launch_pdl_split(ctx->pme, !d_q ? k_colsort<kPackNone> : (host_in ? k_colsort<kPackAtomT> : k_colsort<kPackGather>),
+        e = launch_pdl_split(pme_beside(ctx), !d_q ? k_colsort<kPackNone> : (host_in ? k_colsort<kPackAtomT> : k_colsort<kPackGather>),
                        dim3(ctx->n_cols), dim3(kSortThreads), 0, st, (const int *)d.col_count + (direct ? 0 : ctx->n_cols + 1),
                        d.col_slot, direct, d.counts, d.col_sys, d.sys, (const int *)d.stage_fix, ctx->col_cap, d.stage,
                        (const int *)d.atom_col, d.wpos, d.xyzq, d.tslot, d.perm, d.inv, d.bb, d.clus_sys, d.zbin,

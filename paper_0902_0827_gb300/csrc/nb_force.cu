@@ -1889,10 +1889,8 @@ static void launch_force_1(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 {
     if constexpr (!DEBUG) {
         if constexpr (RAD != 2) {
-            const int64_t units = kListSegs * ctx->clus_cap;
-            const bool rounds = !beside_pme && ctx->tune.blocks_per_sm >= 3 &&
-                                units >= (int64_t)kMinRounds * 32 * ctx->num_sms;
-            if (rounds && force1_resident<4, 8, RAD, VIRIAL, DEBUG>(ctx) >= 8)
+            const bool fill = !beside_pme && ctx->tune.blocks_per_sm >= 3 && force_rounds(ctx) >= kMinRounds;
+            if (fill && force1_resident<4, 8, RAD, VIRIAL, DEBUG>(ctx) >= 8)
                 return launch_force_1w<4, 8, RAD, VIRIAL, DEBUG>(ctx, A, beside_pme);
         }
         const bool fours = beside_pme || ctx->tune.blocks_per_sm > 1;
@@ -2043,10 +2041,10 @@ cudaError_t launch_forces_packed(nb_ctx *ctx, float *d_F, double *d_energy, doub
         const long long *pf = pme ? pme_forces_acc(ctx) : nullptr, *ps = pme ? pme_sums_acc(ctx) : nullptr;
         const double pself = pme ? pme_self_coef(ctx) : 0.0;
         if (virial)
-            launch_pdl_split(ctx->pme, k_unpack_forces<true>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc, d_F,
+            launch_pdl_split(pme_beside(ctx), k_unpack_forces<true>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc, d_F,
                        d.xyzq, d.atom_sys, d.sys_acc, ctx->n_sys, en, vi, pf, ps, pself);
         else
-            launch_pdl_split(ctx->pme, k_unpack_forces<false>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc,
+            launch_pdl_split(pme_beside(ctx), k_unpack_forces<false>, dim3(blocks), dim3(tb), 0, ctx->stream, S, d.counts, d.inv, d.facc,
                        d_F, d.xyzq, d.atom_sys, d.sys_acc, ctx->n_sys, en, vi, pf, ps, pself);
     }
     return cudaGetLastError();

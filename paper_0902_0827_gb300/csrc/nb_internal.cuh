@@ -311,6 +311,26 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return launch_pdl_split(false, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
+// Work units of the one-cluster force kernel per warp of a grid that fills the
+// SMs with 32 warps.
+inline int64_t force_rounds(const nb_ctx *ctx) { return kListSegs * ctx->clus_cap / (32 * ctx->num_sms); }
+
+// Whether the PME chain is to share the SMs with the list and force kernels: then
+// all kernels of a step ask for the same shared-memory split, the force kernel's
+// blocks are not let in before the lists are done, and its grid leaves room.  Not
+// for large systems, where each kernel fills the SMs by itself: the room left
+// makes the force kernel, which is most of the step, longer, and the split takes
+// the L1 that tables are read through.  Shared and not, us a step: 311 and 324 at
+// 90,000 atoms, 408 and 407 at 120,000, 540 and 537 at 165,000, 641 and 630 at
+// 200,001, 2,826 and 2,553 at 999,999; with tables 184 and 195 at 39,999, 264 and
+// 264 at 60,000, 386 and 374 at 90,000, 610 and 560 at 150,000, 3,609 and 3,095 at
+// 999,999.
+constexpr int kShareRounds = 16, kShareRoundsTab = 7;
+inline bool pme_beside(const nb_ctx *ctx)
+{
+    return ctx->pme && force_rounds(ctx) < (ctx->tab_n > 0 ? kShareRoundsTab : kShareRounds);
+}
+
 // i-group slots for a context: every column's clusters form groups of
 // `group` clusters, the last one partial, so at most NC / group + C; the
 // capacity covers every supported group size (groups of one cluster: NC).

@@ -842,7 +842,7 @@ static cudaError_t launch_bonded(nb_ctx *ctx, cudaStream_t st, const float *d_po
     const int terms = M.nb + M.na + M.nd;
     if (terms == 0) return cudaSuccess;
     const int blocks = std::max(1, std::min((terms + 255) / 256, 4 * ctx->num_sms));
-    return launch_pdl_split(ctx->pme, k_md_bonded, dim3(blocks), dim3(256), 0, st, M.nb, M.na, M.nd,
+    return launch_pdl_split(pme_beside(ctx), k_md_bonded, dim3(blocks), dim3(256), 0, st, M.nb, M.na, M.nd,
                       (const int2 *)M.bonds, (const float2 *)M.bond_p, (const int4 *)M.angles,
                       (const float2 *)M.angle_p, (const int4 *)M.dihedrals, (const float4 *)M.dihedral_p, d_pos,
                       box_of(ctx), M.bacc, M.acc);
@@ -869,10 +869,11 @@ static cudaError_t md_forces(nb_ctx *ctx, const float *d_pos, const float *d_q, 
         if (e == cudaSuccess) e = cudaEventRecord(M.bjoin, M.bside);
     }
     if (e == cudaSuccess && pme) e = launch_pme_fork(ctx, d_pos, d_q, sums, true);
-    if (e == cudaSuccess) e = launch_build_lists(ctx, pme);
+    if (e == cudaSuccess) e = launch_build_lists(ctx, pme_beside(ctx));
     if (e != cudaSuccess) return abandon_build(ctx, e);
     ctx->built = true;
-    e = launch_forces_packed(ctx, unpack ? M.Fnb : nullptr, unpack ? M.enb : nullptr, nullptr, false, pme, pme);
+    e = launch_forces_packed(ctx, unpack ? M.Fnb : nullptr, unpack ? M.enb : nullptr, nullptr, false, pme,
+                             pme_beside(ctx));
     if (e != cudaSuccess) return e;
     if (pme) return bside ? cudaStreamWaitEvent(ctx->stream, M.bjoin, 0) : cudaSuccess;
     return launch_bonded(ctx, ctx->stream, d_pos);
@@ -1055,14 +1056,14 @@ extern "C" nb_status nb_md_step(nb_ctx *ctx, float *d_pos, float *d_vel, const f
     if (binned) e = ready_histogram(ctx);
     for (int s = 0; s < n_steps && e == cudaSuccess; ++s) {
         if (s == 0)
-            e = launch_pdl_split(ctx->pme, k_md_first, dim3(ib), dim3(64), 0, st, A, bin);
+            e = launch_pdl_split(pme_beside(ctx), k_md_first, dim3(ib), dim3(64), 0, st, A, bin);
         else
-            e = launch_pdl_split(ctx->pme, k_md_between, dim3(ib), dim3(64), 0, st, A, Nb, M.bacc, bin);
+            e = launch_pdl_split(pme_beside(ctx), k_md_between, dim3(ib), dim3(64), 0, st, A, Nb, M.bacc, bin);
         // the half-steps read the short-range sums themselves (no unpack kernel)
         if (e == cudaSuccess) e = md_forces(ctx, d_pos, d_q, d_type, d_energy && s == n_steps - 1, false, binned);
     }
     if (e == cudaSuccess && n_steps > 0)
-        e = launch_pdl_split(ctx->pme, k_md_second, dim3(ib), dim3(64), 0, st, A, Nb, M.bacc,
+        e = launch_pdl_split(pme_beside(ctx), k_md_second, dim3(ib), dim3(64), 0, st, A, Nb, M.bacc,
                              (const long long *)ctx->d.sys_acc, ctx->pme ? pme_sums_acc(ctx) : nullptr,
                              ctx->pme ? pme_self_coef(ctx) : 0.0, d_energy);
     return e == cudaSuccess ? NB_OK : NB_ERR_CUDA;

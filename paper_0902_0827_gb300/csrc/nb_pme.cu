@@ -785,7 +785,7 @@ static cudaError_t launch_corr(nb_ctx *ctx, const float *d_pos, const float *d_q
     const int S = (int)ctx->slot_cap, ct = 128;
     const int cb = std::max(1, std::min((S * kCorrLanes + ct - 1) / ct, 32 * ctx->num_sms));
     const cudaError_t e =
-        launch_pdl_split(true, k_pme_corr, dim3(cb), dim3(ct), 0, P.cside, P.c, S, (const int *)d.counts,
+        launch_pdl_split(pme_beside(ctx), k_pme_corr, dim3(cb), dim3(ct), 0, P.cside, P.c, S, (const int *)d.counts,
                          (const int *)d.perm, (const int *)d.inv, (const float4 *)d.xyzq, d_pos, d_q,
                          (const int *)d.part_orig, ctx->K, sums ? 1 : 0, P.pacc, P.acc, d.status);
     return e == cudaSuccess ? cudaEventRecord(P.corr, P.cside) : e;
@@ -801,7 +801,7 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     auto &d = ctx->d;
     const dim3 sgrid(g.K1, (g.K2 + g.Ty - 1) / g.Ty);
     const size_t smem = 2 * sizeof(int) * g.Ty * g.K3;
-    cudaError_t e = launch_pdl_split(true, packed ? k_pme_spread<N, true> : k_pme_spread<N, false>, sgrid, dim3(kPmeThreads), smem, st, g,
+    cudaError_t e = launch_pdl_split(pme_beside(ctx), packed ? k_pme_spread<N, true> : k_pme_spread<N, false>, sgrid, dim3(kPmeThreads), smem, st, g,
                                      (const SysDesc *)d.sys, (const int *)d.col_slot, (const float4 *)d.xyzq,
                                      (const int *)d.perm, d_q, P.grid);
     if (e == cudaSuccess) e = launch_corr(ctx, d_pos, d_q, sums);
@@ -812,7 +812,7 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     const float a = ctx->pp.alpha;
     const float pi2_over_a2 = (float)(M_PI * M_PI / ((double)a * (double)a));
     const int sb = std::max(1, std::min((half + 255) / 256, 2 * ctx->num_sms));
-    e = launch_pdl_split(true, k_pme_solve, dim3(sb), dim3(256), 0, st, half, g, pi2_over_a2, (const float *)P.gfac,
+    e = launch_pdl_split(pme_beside(ctx), k_pme_solve, dim3(sb), dim3(256), 0, st, half, g, pi2_over_a2, (const float *)P.gfac,
                          P.fq, P.acc);
     if (e != cudaSuccess) return e;
     e = cudaStreamWaitEvent(st, P.corr, 0);
@@ -823,7 +823,7 @@ static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos
     const int S = (int)ctx->slot_cap;
     const int gt = 256;
     const int gb = std::max(1, std::min((S * G + gt - 1) / gt, 16 * ctx->num_sms));
-    return launch_pdl_split(true, k_pme_gather<N>, dim3(gb), dim3(gt), 0, st, g, S, (const int *)d.counts,
+    return launch_pdl_split(pme_beside(ctx), k_pme_gather<N>, dim3(gb), dim3(gt), 0, st, g, S, (const int *)d.counts,
                             (const int *)d.perm, (const float4 *)d.xyzq, d_q, (const float *)P.grid, P.pacc);
 }
 

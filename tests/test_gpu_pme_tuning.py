@@ -41,3 +41,20 @@ def test_every_grid_gives_the_same_step(group, split, n_types):
             ctx.status()
             for x, y in zip(got, want):
                 assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("n_waters,tables", [(18001, 1024), (25001, 1024), (45001, 0), (66667, 0)])
+def test_both_sides_of_the_line_between_shared_and_full_grids(n_waters, tables):
+    s = S.water_box(n_waters=n_waters)
+    ctx = nb.Nonbonded(s)
+    ctx.set_tables(tables)
+    ctx.set_pme((64, 64, 64), 4)
+    pos, q, t = nb.concat_inputs([s])
+    ctx.build(pos)
+    want = [x.clone() for x in ctx.forces(pos, q, t)]
+    for _ in range(3):
+        got = ctx.step(pos, q, t)
+        torch.cuda.synchronize()
+        ctx.status()
+        for x, y in zip(got, want):
+            assert torch.equal(x, y)
