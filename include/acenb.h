@@ -120,7 +120,8 @@ typedef struct {
 /* nb_create - one system.  Copies params, validates them (box/cutoff ratio,
  * index ranges, disjoint topology), allocates all device scratch and binds
  * the context to `cuda_stream` (a cudaStream_t; NULL = legacy default).
- * Errors: NB_ERR_INVALID_ARG, NB_ERR_BOX_TOO_SMALL, NB_ERR_UNSUPPORTED,
+ * Errors: NB_ERR_INVALID_ARG, NB_ERR_BOX_TOO_SMALL, NB_ERR_UNSUPPORTED (also
+ * for more atoms than 25 bits can number 8-atom clusters of, about 2^28),
  * NB_ERR_OOM, NB_ERR_CUDA.  *out is NULL on error. */
 nb_status nb_create(const nb_params *params, void *cuda_stream, nb_ctx **out);
 
@@ -135,7 +136,8 @@ nb_status nb_create_batch(int32_t n_sys, const nb_params *params, void *cuda_str
  * cluster bounding boxes, map exclusions to the sorted order and build the
  * cluster-pair list (section "Molecular dynamics on the GPU", cell-list
  * construction).  Asynchronous.  Device errors: NB_ERR_NONFINITE,
- * NB_ERR_CAPACITY. */
+ * NB_ERR_CAPACITY.  After a build that returned NB_ERR_CUDA (here, in nb_step
+ * or in an MD step) nb_forces returns NB_ERR_NOT_BUILT until the next one. */
 nb_status nb_build_cells(nb_ctx *ctx, const float *d_pos);
 
 /* nb_forces - forces, energies and virial for the positions of the last

@@ -183,9 +183,11 @@ __device__ void bitonic_sort(unsigned long long *skey, int P)
 // flight with its other first loads) and the list kernel zeroes the
 // histogram; above, the last block of the binning kernel scans the histogram
 // once (the blocks' loads grow with the square of the columns).  Rebuild +
-// forces with the scan and without: 82.5 and 79.9 us at 23,500 atoms (196
+// forces with the scan and without: 82.5 and 79.4 us at 23,500 atoms (196
 // columns), 45.4 and 43.0 us at 6,144, 933 and 914 us for 64 boxes (4,508
-// columns), 1991 and 1977 us at 999,999 (2,401).
+// columns), 1991 and 1976 us at 999,999 (2,401).  Towards the line the gain
+// still grows: 98 and 81 us for a thin gas of 4,489 columns, 128 and 106 for
+// 6,241, 529 and 507 for a slab of 6,561, 764 and 738 for 500 boxes of 16.
 constexpr int kDirectCols = 8192;
 constexpr int kRankSortMax = 256;  // columns up to this many atoms are rank-sorted (no barriers)
 
@@ -624,7 +626,7 @@ __device__ __forceinline__ int div_small(int a, int b, float inv_b, int &r)
 struct GListArgs {
     const SysDesc *sys;
     const int *counts;
-    int *pool_count;         // pool records used (counts[5], zeroed by the binning kernel)
+    int *pool_count;         // pool records used (counts[5], zeroed by the column sort or the binning kernel's scan)
     const float4 *bb;
     const int *clus_sys;
     const int *col_slot;
@@ -937,9 +939,9 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
     }
 }
 
-// A4 for groups of one cluster (the default tile shape): the lists and masks
-// of k_glist with group = 1, entry for entry, by a kernel that uses what one
-// cluster allows.
+// A4 for groups of one cluster (the default tile shape): the entries that
+// k_glist would list with group = 1, in the same order, by a kernel that uses
+// what one cluster allows.
 //
 // * Half of the candidates are never looked at.  keep_groups keeps J > g when
 //   the indices differ in parity and J < g when they share it, and the
@@ -954,16 +956,16 @@ __global__ void __launch_bounds__(kGListWarps * 32, ACENB_GLIST_MIN_BLOCKS) k_gl
 //
 // Bound by the instructions of each warp's dependent chain: at 23,500 atoms
 // the groups are one wave of 20 warps per SM.  Against k_glist for the same
-// lists: rebuild + forces 85.6 -> 83.0 us at 23,500 atoms, 48.6 -> 46.2 us at
-// 6,144, 2129 -> 1988 us at 999,999.  64 registers (8 blocks per SM): 72 cost
+// lists: rebuild + forces 85.6 -> 82.6 us at 23,500 atoms, 48.6 -> 46.4 us at
+// 6,144, 2129 -> 1982 us at 999,999.  64 registers (8 blocks per SM): 72 cost
 // 22 us at 999,999 atoms, 56 gain 6 us there and cost 1 us at 23,500.
 constexpr int kGList1MinBlocks = 8;
 constexpr int kMapWords = 32;  // partner-cluster map: 1,024 bits
 
-// BESIDE: as for k_glist.  (With the equal shared-memory split of launch_pdl_split:
-// rebuild + forces with PME 125.5 -> 113.3 us at 23,500 atoms, the MD step
-// 127 -> 114 us; without the second force launch that used to follow the PME
-// chain, 109 and 106 us.)
+// BESIDE: as for k_glist.  (With the equal shared-memory split of
+// launch_pdl_split, and without a second force launch behind the PME chain:
+// rebuild + forces with PME 127.2 -> 109.4 us at 23,500 atoms, ten MD steps
+// 1299 -> 1060.)
 template <bool BESIDE>
 __global__ void __launch_bounds__(kGListWarps * 32, kGList1MinBlocks) k_glist1(GListArgs A)
 {

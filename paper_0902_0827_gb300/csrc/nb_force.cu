@@ -320,8 +320,9 @@ __device__ __forceinline__ void record_pair(const ForceArgs &A, int io, int jo)
 }
 
 // Tile fill counters of the debug instantiation: tiles visited (dbg_n[3])
-// and tile halves whose radial arithmetic runs (dbg_n[2]); with the pair
-// count they give the fraction of evaluated lanes inside the cutoff.
+// and tile halves with a pair in range (dbg_n[2]), the halves whose arithmetic
+// runs in k_force<G> (k_force1 evaluates both halves of a tile with a pair);
+// with the pair count they give the fill of the tiles and of those halves.
 __device__ __forceinline__ void count_tile(const ForceArgs &A, bool anyA, bool anyB)
 {
     if ((threadIdx.x & 31) == 0) {
@@ -785,7 +786,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, ACENB_TILE_MIN_BLOCKS) k_forc
 // A tile with a pair in range is evaluated whole; voting on its two halves
 // and skipping one (scalar code, 1.35 halves per tile) took 47.9 M warp
 // instructions and 63.4 us per launch at 23,500 atoms and 1,661 us at
-// 999,999; packed it is 40.3 M, 60.8 us and 1,621 us.  (An FMA with three
+// 999,999; packed it was 40.3 M, 60.8 us and 1,621 us, and with the unit claims
+// and block shapes below it is 39.7 M, 57.0 us and 1,569 us.  (An FMA with three
 // register operands, packed or not, issues at about 0.6 of its rate for the
 // register reads: the constants of the polynomials come from the parameter
 // bank and run at the full rate.)
@@ -1866,8 +1868,8 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 
 // Which instance.  Blocks of 4 warps start and end in smaller steps than
 // blocks of 8 (the kernel before and the kernel after share the SM's registers
-// with them sooner): rebuild + forces 93.4 -> 90.6 us at 23,500 atoms,
-// 53.2 -> 51.2 us at 6,144.  Each block holds the type-pair table, so with many
+// with them sooner): rebuild + forces, with the unit claims as they are now,
+// 93.4 -> 90.6 us at 23,500 atoms, 53.2 -> 51.2 us at 6,144.  Each block holds the type-pair table, so with many
 // types (above about 26) an SM holds fewer warps in blocks of 4 than in blocks
 // of 8, and blocks of 8 are taken.  So are they for a grid of 8 warps per SM
 // (blocks_per_sm 1), whose blocks of 4 would not spread evenly over SMs that
@@ -1878,7 +1880,8 @@ static void launch_force_1w(nb_ctx *ctx, const ForceArgs &A, bool beside_pme)
 // blocks_per_sm 2, 2,307 with 80 registers), pays once every warp has kMinRounds
 // units (the longer units of fuller SMs make the end of a launch longer):
 // 1976 -> 1928 us at 999,999 atoms, 511 -> 503 at 240,000, 914 -> 903 for 64
-// boxes, 110.7 -> 109.2 at 39,003, but 90.6 -> 93.1 us at 23,500.  The
+// boxes, 110.7 -> 109.2 at 39,003, but 90.6 -> 93.1 us at 23,500 (all water: an
+// SM has to hold 8 blocks with their tables, so up to 17 types).  The
 // tabulated form does not take it: 80.9 -> 83.3 us at 20,001 atoms, 129.0 ->
 // 131.9 at 39,003, 262 -> 268 at 90,000 (its loads go to L1 and L2, which more
 // warps share).
@@ -2114,8 +2117,8 @@ cudaError_t launch_adjoint_tile(nb_ctx *ctx, const double *d_dLdE, float *d_dpos
 }
 
 // Test export of the pair arithmetic (nb_debug_pair_terms): pair k of the
-// given lists evaluated by eval_pair exactly as the forward kernel does it
-// (unit weights, d = x_j - x_i as given); out[2k] = (E_LJ, E_Coul, r2, 0),
+// given lists evaluated by eval_pair, as k_force<G> does it (k_force1's packed
+// form has the same bits; unit weights, d = x_j - x_i as given); out[2k] = (E_LJ, E_Coul, r2, 0),
 // out[2k + 1] = the force on j.
 template <int RAD>
 __global__ void k_debug_pair_terms(PairParams P, const float4 *__restrict__ lj_tab, const float4 *__restrict__ rtab,

@@ -168,7 +168,7 @@ struct DevBuffers {
     float4 *rtab = nullptr;          // [tab_n*3] tabulated radial functions (nb_set_tables)
     float4 *gslot = nullptr;         // [S] adjoint input dL/dF in sorted order
     float *eps_type = nullptr;       // [T] per-type epsilon (Lorentz-Berthelot chain)
-    long long *dbg_n = nullptr;      // [4] debug counters: pair evaluations, pairs, evaluated tile halves, tiles
+    long long *dbg_n = nullptr;      // [4] debug counters: pair evaluations, pairs, tile halves with a pair, tiles
     int *dbg_ij = nullptr;           // [cap*2]
     int64_t dbg_cap = 0;
     float *scratch_f = nullptr;      // [N*3] debug force sink
@@ -285,7 +285,7 @@ __device__ __forceinline__ void pdl_entry()
 // with the largest shared-memory carve-out.  An SM changes its split between
 // L1 and shared memory only when it is empty, so kernels that are to share
 // SMs with the force kernel, which needs most of it, have to run with the same
-// split (the steps with PME, where two chains run side by side).
+// split (the steps with PME whose two chains run side by side: pme_beside).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_split(bool shared, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                              Args &&...args)

@@ -792,7 +792,10 @@ static cudaError_t launch_corr(nb_ctx *ctx, const float *d_pos, const float *d_q
 }
 
 // The grid's chain on stream st; the corrections are launched behind the
-// spread (whose blocks go first where both fit), the gather waits for them.
+// spread (whose blocks go first where both fit) and waited for before the
+// inverse transform: a wait between it and the gather would keep the gather's
+// blocks from coming in early (nb_pme_forces of order 6 at 6,144 atoms 61.0 us
+// with the wait there, 58.7 here).
 template <int N>
 static cudaError_t launch_pme_t(nb_ctx *ctx, cudaStream_t st, const float *d_pos, const float *d_q, bool sums, bool packed)
 {
@@ -954,7 +957,7 @@ extern "C" nb_status nb_set_pme(nb_ctx *ctx, const nb_pme_params *p)
     if (e == cudaSuccess) e = cudaMalloc(&P->pacc, sizeof(long long) * 3 * std::max<int64_t>(ctx->slot_cap, 1));
     if (e == cudaSuccess) e = cudaMalloc(&P->acc, sizeof(long long) * kPmeAcc);
     if (e == cudaSuccess) e = cudaMemset(P->acc, 0, sizeof(long long) * kPmeAcc);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->cside, cudaStreamNonBlocking);

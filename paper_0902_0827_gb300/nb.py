@@ -473,7 +473,7 @@ class Nonbonded:
         return ij[order], n.value, no.value
 
     def debug_fill(self):
-        """(tiles visited, tile halves evaluated) of the last debug_pairs run."""
+        """(tiles visited, tile halves with a pair in range) of the last debug_pairs run."""
         t, h = ctypes.c_int64(), ctypes.c_int64()
         _check(lib().nb_debug_fill(self.h, ctypes.byref(t), ctypes.byref(h)), "nb_debug_fill")
         return t.value, h.value
