@@ -1253,6 +1253,22 @@ bool bins_elsewhere(nb_ctx *ctx, const float *d_q)
     return ctx->n_sys == 1 && ctx->n_cols <= kDirectCols && !inputs_in_host_memory(ctx, d_q);
 }
 
+static bool capturing(const nb_ctx *ctx)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(ctx->stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
+}
+
+// (A captured clearing runs with its graph: a call before that clears too.)
+static cudaError_t clear_histogram(nb_ctx *ctx)
+{
+    const cudaError_t e =
+        cudaMemsetAsync(ctx->d.col_count, 0, sizeof(int) * (2 * (size_t)ctx->n_cols + 1), ctx->stream);
+    if (e != cudaSuccess) ctx->hist_dirty = true;
+    else if (!capturing(ctx)) ctx->hist_dirty = false;
+    return e;
+}
+
 // A second set of counts on top of the first would overflow the sorted arrays
 // (every atom staged twice), so the counts of a build whose lists were not
 // launched are cleared at once, in stream order: a graph captured earlier finds
@@ -1265,23 +1281,14 @@ bool bins_elsewhere(nb_ctx *ctx, const float *d_q)
 cudaError_t abandon_build(nb_ctx *ctx, cudaError_t e)
 {
     cudaGetLastError();
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs == cudaStreamCaptureStatusNone) ctx->built = false;
+    if (!capturing(ctx)) ctx->built = false;
     if (ctx->pme) pme_rejoin(ctx);
-    ctx->hist_dirty = cudaMemsetAsync(ctx->d.col_count, 0, sizeof(int) * (2 * (size_t)ctx->n_cols + 1), ctx->stream) !=
-                      cudaSuccess;
+    clear_histogram(ctx);
     cudaGetLastError();
     return e;
 }
 
-cudaError_t ready_histogram(nb_ctx *ctx)
-{
-    if (!ctx->hist_dirty) return cudaSuccess;
-    const cudaError_t e =
-        cudaMemsetAsync(ctx->d.col_count, 0, sizeof(int) * (2 * (size_t)ctx->n_cols + 1), ctx->stream);
-    ctx->hist_dirty = e != cudaSuccess;
-    return e;
-}
+cudaError_t ready_histogram(nb_ctx *ctx) { return ctx->hist_dirty ? clear_histogram(ctx) : cudaSuccess; }
 
 cudaError_t launch_build_cells(nb_ctx *ctx, const float *d_pos, const float *d_q, const int32_t *d_type, bool binned)
 {
